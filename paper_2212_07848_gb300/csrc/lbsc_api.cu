@@ -32,6 +32,7 @@ struct lb_ctx {
     double *d_out = nullptr;        // small device results (conserved sums, bins)
     int nred = 0;
     double *d_io = nullptr;         // nx*ny doubles for density / read-outs (lazy)
+    HostReadout rd;                 // radial bins, moments and the flag (lazy, host memory)
     // structure factor (lazy, powers of two only)
     void *drho = nullptr;
     void *spec = nullptr;
@@ -216,6 +217,7 @@ void free_all(lb_ctx *h) {
     cudaFree(h->d_partials);
     cudaFree(h->d_out);
     cudaFree(h->d_io);
+    h->rd.release();
     cudaFree(h->drho);
     cudaFree(h->spec);
     cudaFree(h->acc);
@@ -682,6 +684,15 @@ int lb_sk_sample_now(lb_ctx *h) {
     return sample_sk(h);
 }
 
+// Wait for a read-out whose kernel wrote its values and the flag to h->rd.
+static int readout_sync(lb_ctx *h) {
+    LB_CHECK(cudaStreamSynchronize(h->stream));
+    const int flag = *(volatile int *)h->rd.flag();
+    if (!flag) return LB_OK;
+    LB_CHECK(cudaMemset(h->d_flag, 0, sizeof(int)));
+    return (flag & LB_STEP_TIMEOUT) ? LB_ERR_TIMEOUT : LB_ERR_NONFINITE;
+}
+
 int lb_structure_factor(lb_ctx *h, double *host_out, int nbins, long long *nsamples_out) {
     if (!h || !host_out || nbins < 0 || nbins > 4096) return LB_ERR_ARG;
     int rc = select_device(h);
@@ -696,18 +707,14 @@ int lb_structure_factor(lb_ctx *h, double *host_out, int nbins, long long *nsamp
         LB_CHECK(cudaMemcpyAsync(host_out, h->d_io, (size_t)(nx / 2 + 1) * ny * sizeof(double),
                                  cudaMemcpyDeviceToHost, h->stream));
     } else {
-        rc = ensure_io(h);
+        LB_CHECK(h->rd.ensure());
+        LB_CHECK(launch_sk_bins(h->acc, inv, h->rd.v, h->d_flag, h->rd.flag(), nbins, nx, ny,
+                                h->ldx, h->stream));
+        rc = readout_sync(h);
         if (rc) return rc;
-        double *bins = h->d_io, *counts = h->d_io + nbins;
-        LB_CHECK(cudaMemsetAsync(h->d_io, 0, 2 * (size_t)nbins * sizeof(double), h->stream));
-        LB_CHECK(launch_sk_bins(h->acc, inv, bins, counts, nbins, nx, ny, h->ldx, h->stream));
-        std::vector<double> tmp(2 * (size_t)nbins);
-        LB_CHECK(cudaMemcpyAsync(tmp.data(), h->d_io, 2 * (size_t)nbins * sizeof(double),
-                                 cudaMemcpyDeviceToHost, h->stream));
-        rc = lb_sync(h);
-        if (rc) return rc;
-        for (int b = 0; b < nbins; ++b)
-            host_out[b] = tmp[nbins + b] > 0 ? tmp[b] / tmp[nbins + b] : NAN;
+        memcpy(host_out, h->rd.v, nbins * sizeof(double));
+        if (nsamples_out) *nsamples_out = h->sk_count;
+        return LB_OK;
     }
     if (nsamples_out) *nsamples_out = h->sk_count;
     return lb_sync(h);
@@ -719,9 +726,14 @@ int lb_sk_moments(lb_ctx *h, double out[2]) {
     if (rc) return rc;
     if (!h->acc) return LB_ERR_STATE;
     const double inv = h->sk_count > 0 ? 1.0 / (double)h->sk_count : 0.0;
-    LB_CHECK(launch_sk_moments(h->acc, inv, h->p.nx, h->p.ny, h->ldx, h->d_out, h->stream));
-    LB_CHECK(cudaMemcpyAsync(out, h->d_out, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    return lb_sync(h);
+    LB_CHECK(h->rd.ensure());
+    LB_CHECK(launch_sk_moments(h->acc, inv, h->p.nx, h->p.ny, h->ldx, h->d_partials, h->nred,
+                               h->rd.v, h->d_flag, h->rd.flag(), h->stream));
+    rc = readout_sync(h);
+    if (rc) return rc;
+    out[0] = h->rd.v[0];
+    out[1] = h->rd.v[1];
+    return LB_OK;
 }
 
 int lb_structure_factor_counts(lb_ctx *h, long long *host_counts, int nbins) {

@@ -331,6 +331,7 @@ struct lb_ens {
     int *d_flag = nullptr;
     double *d_io = nullptr, *d_partials = nullptr, *d_out = nullptr;
     size_t io_elems = 0;
+    HostReadout rd;                     // radial bins and the flag (lazy, host memory)
     int nred = 0;
     EnsKeys keys;
     long long t = 0;
@@ -724,6 +725,7 @@ void free_ens(lb_ens *e) {
     cudaFree(e->d_clk);
     cudaFree(e->d_flag);
     cudaFree(e->d_io);
+    e->rd.release();
     cudaFree(e->d_partials);
     cudaFree(e->d_out);
     cudaFree(e->d_nbr_off);
@@ -1123,16 +1125,16 @@ int lb_ens_structure_factor(lb_ens *e, int r, double *host_out, int nbins,
         rc = ens_sync(e);
         if (rc) return rc;
     } else {
-        ENS_CHECK(cudaMemsetAsync(e->d_io, 0, 2 * (size_t)nbins * sizeof(double), e->stream));
-        ENS_CHECK(launch_sk_bins(R.acc, inv, e->d_io, e->d_io + nbins, nbins, R.nx, R.ny, R.ldx,
-                                 e->stream));
-        std::vector<double> tmp(2 * (size_t)nbins);
-        ENS_CHECK(cudaMemcpyAsync(tmp.data(), e->d_io, tmp.size() * sizeof(double),
-                                  cudaMemcpyDeviceToHost, e->stream));
-        rc = ens_sync(e);
-        if (rc) return rc;
-        for (int b = 0; b < nbins; ++b)
-            host_out[b] = tmp[nbins + b] > 0 ? tmp[b] / tmp[nbins + b] : NAN;
+        ENS_CHECK(e->rd.ensure());
+        ENS_CHECK(launch_sk_bins(R.acc, inv, e->rd.v, e->d_flag, e->rd.flag(), nbins, R.nx, R.ny,
+                                 R.ldx, e->stream));
+        ENS_CHECK(cudaStreamSynchronize(e->stream));
+        const int flag = *(volatile int *)e->rd.flag();
+        if (flag) {
+            ENS_CHECK(cudaMemset(e->d_flag, 0, sizeof(int)));
+            return (flag & LB_STEP_TIMEOUT) ? LB_ERR_TIMEOUT : LB_ERR_NONFINITE;
+        }
+        memcpy(host_out, e->rd.v, nbins * sizeof(double));
     }
     if (nsamples_out) *nsamples_out = e->sk_count;
     return LB_OK;

@@ -78,10 +78,32 @@ cudaError_t launch_sk_sample(int precision, const SkArgs &a, cudaStream_t s);
 cudaError_t launch_twiddles(int precision, void *tw, int n, cudaStream_t s);
 cudaError_t launch_sk_readout(const double *acc, double inv_count, double *out, int nx,
                               int ny, int ldx, cudaStream_t s);
-cudaError_t launch_sk_bins(const double *acc, double inv_count, double *bins, double *counts,
-                           int nbins, int nx, int ny, int ldx, cudaStream_t s);
+// Radial means of the first nbins bins (NaN where empty) into out and the status
+// flag into flag_out (both device-visible; host memory mapped into the device
+// saves the copy back).
+cudaError_t launch_sk_bins(const double *acc, double inv_count, double *out, const int *flag,
+                           int *flag_out, int nbins, int nx, int ny, int ldx, cudaStream_t s);
+// part: 2 nblocks doubles of scratch.
 cudaError_t launch_sk_moments(const double *acc, double inv_count, int nx, int ny, int ldx,
-                              double *out2, cudaStream_t s);
+                              double *part, int nblocks, double *out2, const int *flag,
+                              int *flag_out, cudaStream_t s);
+
+// Small host buffer mapped into the device, which read-out kernels write
+// directly (the values and the status flag); allocated on first use.
+constexpr int kReadoutMax = 4096;
+struct HostReadout {
+    double *v = nullptr;   // [kReadoutMax], then the flag
+    int *flag() const { return reinterpret_cast<int *>(v + kReadoutMax); }
+    cudaError_t ensure() {
+        if (v) return cudaSuccess;
+        return cudaHostAlloc((void **)&v, (kReadoutMax + 1) * sizeof(double),
+                             cudaHostAllocMapped | cudaHostAllocPortable);
+    }
+    void release() {
+        if (v) cudaFreeHost(v);
+        v = nullptr;
+    }
+};
 cudaError_t launch_conserved(int precision, const void *df, double *partials, int nblocks,
                              double *out3, int nx, int ny, cudaStream_t s);
 int conserved_blocks(int nx, int ny);
