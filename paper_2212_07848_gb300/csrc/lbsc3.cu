@@ -448,72 +448,117 @@ step3_kernel(const K3<T> p) {
 
 // ---------------------------------------------------------------------------
 // Axis structure factor: per z plane the partial x and y profiles of delta
-// rho and the plane total; then the profiles are summed over planes in a
-// fixed order and Fourier transformed on the x, y and z axes.
+// rho and the plane total (one read of the sample); the profiles summed over
+// planes in a fixed order; and a warp per axis mode for its Fourier sum.
+// 256^3: 161 + 9 + 19 us for the three, against 228 us (three reads of each
+// plane by one block) and 1164 us (one block for the sums and all 384 modes,
+// bound by the FP64 sine and cosine of every term on a single SM).
 // ---------------------------------------------------------------------------
+template <typename T> struct Vec4;
+template <> struct Vec4<float> { using t = float4; };
+template <> struct Vec4<double> { using t = double4; };
+
+constexpr int kProfWarps = 8;
+
+// Block = one z plane; warp w takes rows w, w + 8, ... in chunks of 128
+// columns, four neighbouring columns to a lane (nx is a multiple of 32).
 template <typename T>
-__global__ void profile3_kernel(const T *__restrict__ drho, int nx, int ny, double *__restrict__ px,
-                                double *__restrict__ py, double *__restrict__ pz) {
-    // block = one z plane
-    const int z = blockIdx.x;
+__global__ void __launch_bounds__(32 * kProfWarps)
+profile3_kernel(const T *__restrict__ drho, int nx, int ny, double *__restrict__ px,
+                double *__restrict__ py, double *__restrict__ pz) {
+    using V = typename Vec4<T>::t;
+    __shared__ double sh[kProfWarps][128];
+    const int z = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const T *pl = drho + (size_t)z * nx * ny;
-    for (int x = threadIdx.x; x < nx; x += blockDim.x) {
-        double s = 0.0;
-        for (int y = 0; y < ny; ++y) s += (double)pl[(size_t)y * nx + x];
-        px[(size_t)z * nx + x] = s;
-    }
-    for (int y = threadIdx.x; y < ny; y += blockDim.x) {
-        double s = 0.0;
-        for (int x = 0; x < nx; ++x) s += (double)pl[(size_t)y * nx + x];
-        py[(size_t)z * ny + y] = s;
-    }
-    __shared__ double red[256];
-    double s = 0.0;
-    for (size_t i = threadIdx.x; i < (size_t)nx * ny; i += blockDim.x) s += (double)pl[i];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+    double *rows = py + (size_t)z * ny;
+    for (int x0 = 0; x0 < nx; x0 += 128) {
+        const int x = x0 + 4 * lane;
+        double c0 = 0.0, c1 = 0.0, c2 = 0.0, c3 = 0.0;
+        for (int y = w; y < ny; y += kProfWarps) {
+            double r = 0.0;
+            if (x < nx) {
+                const V v = *reinterpret_cast<const V *>(pl + (size_t)y * nx + x);
+                const double a = (double)v.x, b = (double)v.y, c = (double)v.z, d = (double)v.w;
+                c0 += a;
+                c1 += b;
+                c2 += c;
+                c3 += d;
+                r = (a + b) + (c + d);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) r += __shfl_down_sync(0xffffffffu, r, o);
+            if (lane == 0) rows[y] = x0 ? rows[y] + r : r;
+        }
+        sh[w][4 * lane] = c0;
+        sh[w][4 * lane + 1] = c1;
+        sh[w][4 * lane + 2] = c2;
+        sh[w][4 * lane + 3] = c3;
         __syncthreads();
+        if (threadIdx.x < 128 && x0 + threadIdx.x < nx) {
+            double v = 0.0;
+            for (int k = 0; k < kProfWarps; ++k) v += sh[k][threadIdx.x];
+            px[(size_t)z * nx + x0 + threadIdx.x] = v;
+        }
+        __syncthreads();   // also: every row sum of this chunk is visible to the block
     }
-    if (threadIdx.x == 0) pz[z] = red[0];
+    if (w == 0) {
+        double v = 0.0;
+        for (int y = lane; y < ny; y += 32) v += rows[y];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        if (lane == 0) pz[z] = v;
+    }
 }
 
-// one block: the profiles are summed over planes in a fixed order into
-// shared memory, then a thread per axis mode accumulates
-// |sum_c p(c) e^{-2 pi i m c / n}|^2 / N.
-__global__ void axis_dft3_kernel(const double *__restrict__ px, const double *__restrict__ py,
-                                 const double *__restrict__ pz, int nx, int ny, int nz,
-                                 double *__restrict__ acc) {
-    extern __shared__ double tot[];   // [nx] + [ny] + [nz]
-    for (int c = threadIdx.x; c < nx; c += blockDim.x) {
-        double v = 0.0;
-        for (int z = 0; z < nz; ++z) v += px[(size_t)z * nx + c];
+// tot[c] = the sum over z planes of profile column c (the nx columns of px,
+// then the ny of py): 32 columns to a block, its warps share the planes.
+__global__ void __launch_bounds__(32 * kProfWarps)
+axis_sum3_kernel(const double *__restrict__ px, const double *__restrict__ py, int nx, int ny,
+                 int nz, double *__restrict__ tot) {
+    __shared__ double sh[kProfWarps][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int c = blockIdx.x * 32 + lane;
+    double v = 0.0;
+    if (c < nx + ny) {
+        const double *col = c < nx ? px + c : py + (c - nx);
+        const size_t ld = c < nx ? nx : ny;
+#pragma unroll 4
+        for (int z = w; z < nz; z += kProfWarps) v += col[(size_t)z * ld];
+    }
+    sh[w][lane] = v;
+    __syncthreads();
+    if (w == 0 && c < nx + ny) {
+        v = 0.0;
+        for (int k = 0; k < kProfWarps; ++k) v += sh[k][lane];
         tot[c] = v;
     }
-    for (int c = threadIdx.x; c < ny; c += blockDim.x) {
-        double v = 0.0;
-        for (int z = 0; z < nz; ++z) v += py[(size_t)z * ny + c];
-        tot[nx + c] = v;
+}
+
+// A warp per axis mode: acc += |sum_c p(c) e^{-2 pi i m c / n}|^2 / N, with
+// tot = the profiles on x and y and pz the one on z.
+__global__ void __launch_bounds__(64)
+axis_dft3_kernel(const double *__restrict__ tot, const double *__restrict__ pz, int nx, int ny,
+                 int nz, double *__restrict__ acc) {
+    const int lane = threadIdx.x & 31, t = (int)(blockIdx.x * 2 + (threadIdx.x >> 5));
+    if (t >= nx / 2 + ny / 2 + nz / 2) return;
+    int m, n;
+    const double *p;
+    if (t < nx / 2) { m = t + 1; n = nx; p = tot; }
+    else if (t < nx / 2 + ny / 2) { m = t - nx / 2 + 1; n = ny; p = tot + nx; }
+    else { m = t - nx / 2 - ny / 2 + 1; n = nz; p = pz; }
+    double re = 0.0, im = 0.0;
+    for (int c = lane; c < n; c += 32) {
+        double sn, cs;
+        sincospi(2.0 * (double)(((long long)m * c) % n) / n, &sn, &cs);
+        re += p[c] * cs;
+        im -= p[c] * sn;
     }
-    for (int c = threadIdx.x; c < nz; c += blockDim.x) tot[nx + ny + c] = pz[c];
-    __syncthreads();
-    const int nmodes = nx / 2 + ny / 2 + nz / 2;
-    const double N = (double)nx * ny * nz;
-    for (int t = threadIdx.x; t < nmodes; t += blockDim.x) {
-        int m, n, off;
-        if (t < nx / 2) { m = t + 1; n = nx; off = 0; }
-        else if (t < nx / 2 + ny / 2) { m = t - nx / 2 + 1; n = ny; off = nx; }
-        else { m = t - nx / 2 - ny / 2 + 1; n = nz; off = nx + ny; }
-        double re = 0.0, im = 0.0;
-        for (int c = 0; c < n; ++c) {
-            double sn, cs;
-            sincospi(2.0 * (double)(((long long)m * c) % n) / n, &sn, &cs);
-            re += tot[off + c] * cs;
-            im -= tot[off + c] * sn;
-        }
-        acc[t] += (re * re + im * im) / N;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        re += __shfl_down_sync(0xffffffffu, re, o);
+        im += __shfl_down_sync(0xffffffffu, im, o);
     }
+    if (lane == 0) acc[t] += (re * re + im * im) / ((double)nx * ny * nz);
 }
 
 template <typename T>
@@ -670,64 +715,157 @@ __global__ void fft_lines_kernel(typename C2<T>::t *__restrict__ data, int n, in
 // Radial bins over the full k cube from the half spectrum: b = round(|q|),
 // q_a = (wave number index on axis a) x max(n) / n_a; a kx column with
 // 0 < kx < nx/2 stands for two modes (k and -k).  k = 0 excluded.
-__global__ void sk3_bins_kernel(const double *__restrict__ acc, double inv_count,
-                                double *__restrict__ bins, double *__restrict__ counts, int nbins,
-                                int nx, int ny, int nz, int ldx) {
-    const int hx = nx / 2 + 1;
-    const size_t total = (size_t)hx * ny * nz;
-    const double L = (double)max(nx, max(ny, nz));
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total;
-         e += (size_t)gridDim.x * blockDim.x) {
-        const int kx = (int)(e % hx);
-        const size_t r = e / hx;
-        const int ky = (int)(r % ny), kz = (int)(r / ny);
-        if (kx == 0 && ky == 0 && kz == 0) continue;
-        const int my = ky <= ny / 2 ? ky : ky - ny, mz = kz <= nz / 2 ? kz : kz - nz;
-        const double qx = (double)kx * (L / nx), qy = (double)my * (L / ny),
-                     qz = (double)mz * (L / nz);
-        const int b = (int)rint(sqrt(qx * qx + qy * qy + qz * qz));
-        if (b >= nbins) continue;
-        const double w = (kx == 0 || 2 * kx == nx) ? 1.0 : 2.0;
-        atomicAdd(&bins[b], w * acc[((size_t)kz * ny + ky) * ldx + kx] * inv_count);
-        atomicAdd(&counts[b], w);
+//
+// The sides are powers of two, so |q|^2 = m is an integer and round(sqrt(m)) =
+// b is exactly b^2 - b < m <= b^2 + b.  Block (b, split) walks the rows (kz, ky)
+// of its share of the planes, a thread a row, and adds the few columns of it
+// inside the shell: no square root, no atomics, a fixed order.  The splits
+// are added by a second launch, which writes the means and the status flag
+// to mapped host memory.  128^3, 112 shells: 33 us for the two against
+// 261 us with an FP64 square root and two atomics per mode.
+constexpr int kBinSplits3 = 16, kBinThreads3 = 128;
+
+__global__ void __launch_bounds__(kBinThreads3)
+sk3_bins_kernel(const double *__restrict__ acc, double *__restrict__ part, int nx, int ny, int nz,
+                int ldx) {
+    const int b = blockIdx.x;
+    const int L = max(nx, max(ny, nz)), sx = L / nx, sy = L / ny, sz = L / nz;
+    double s = 0.0;
+    int cnt = 0;
+    if (b < 20000) {   // the largest |q| is sqrt(3) 8192
+        const int lo2 = b * b - b + 1, hi2 = b * b + b;
+        for (int kz = blockIdx.y; kz < nz; kz += kBinSplits3) {
+            const int qz = min(kz, nz - kz) * sz;
+            if (qz * qz > hi2) continue;
+            for (int ky = threadIdx.x; ky < ny; ky += kBinThreads3) {
+                const int qy = min(ky, ny - ky) * sy, r2 = qz * qz + qy * qy;
+                if (r2 > hi2) continue;
+                const double *row = acc + ((size_t)kz * ny + ky) * ldx;
+                int kx = 0;
+                if (lo2 > r2) {   // the least kx with (kx sx)^2 + r2 >= lo2
+                    kx = (int)(sqrtf((float)(lo2 - r2)) / (float)sx);
+                    while (kx * sx * (kx * sx) + r2 < lo2) ++kx;
+                    while (kx > 0 && (kx - 1) * sx * ((kx - 1) * sx) + r2 >= lo2) --kx;
+                }
+                for (; kx <= nx / 2 && kx * sx * (kx * sx) + r2 <= hi2; ++kx) {
+                    const bool once = kx == 0 || 2 * kx == nx;
+                    s += once ? row[kx] : 2.0 * row[kx];
+                    cnt += once ? 1 : 2;
+                }
+            }
+        }
+    }
+    __shared__ double sh[kBinThreads3 / 32];
+    __shared__ int shc[kBinThreads3 / 32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        s += __shfl_down_sync(0xffffffffu, s, o);
+        cnt += __shfl_down_sync(0xffffffffu, cnt, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        sh[threadIdx.x >> 5] = s;
+        shc[threadIdx.x >> 5] = cnt;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < kBinThreads3 / 32; ++w) {
+            s += sh[w];
+            cnt += shc[w];
+        }
+        double *o = part + 2 * ((size_t)blockIdx.y * gridDim.x + b);
+        o[0] = s;
+        o[1] = (double)cnt;
     }
 }
 
+__global__ void sk3_bins_final_kernel(const double *__restrict__ part, double inv_count, int nbins,
+                                      double *__restrict__ out, const int *__restrict__ flag,
+                                      int *__restrict__ flag_out) {
+    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    if (b == 0) *flag_out = *flag;
+    if (b >= nbins) return;
+    double s = 0.0, cnt = 0.0;
+    for (int k = 0; k < kBinSplits3; ++k) {
+        s += part[2 * ((size_t)k * nbins + b)];
+        cnt += part[2 * ((size_t)k * nbins + b) + 1];
+    }
+    out[b] = cnt > 0.0 ? s * inv_count / cnt : 0.0;
+}
+
 // (sum_k S(k), sum_k |k| S(k)) over the full k cube, k = 0 excluded, |k| =
-// 2 pi sqrt((kx/nx)^2 + (ky/ny)^2 + (kz/nz)^2) with folded indices.  One
-// block, fixed summation order.
-__global__ void __launch_bounds__(256)
-sk3_moments_kernel(const double *__restrict__ acc, double inv_count, int nx, int ny, int nz,
-                   int ldx, double *__restrict__ out) {
-    const int hx = nx / 2 + 1;
-    const size_t total = (size_t)hx * ny * nz;
-    double s0 = 0.0, s1 = 0.0;
-    for (size_t e = threadIdx.x; e < total; e += blockDim.x) {
-        const int kx = (int)(e % hx);
-        const size_t r = e / hx;
-        const int ky = (int)(r % ny), kz = (int)(r / ny);
-        if (kx == 0 && ky == 0 && kz == 0) continue;
-        const int my = ky <= ny / 2 ? ky : ky - ny, mz = kz <= nz / 2 ? kz : kz - nz;
-        const double w = (kx == 0 || 2 * kx == nx) ? 1.0 : 2.0;
-        const double S = acc[((size_t)kz * ny + ky) * ldx + kx] * inv_count;
-        const double qx = (double)kx / nx, qy = (double)my / ny, qz = (double)mz / nz;
-        s0 += w * S;
-        s1 += w * S * 6.283185307179586 * sqrt(qx * qx + qy * qy + qz * qz);
+// 2 pi sqrt((kx/nx)^2 + (ky/ny)^2 + (kz/nz)^2) with folded indices.  Two passes
+// with a fixed order: warps over the rows (mz, my) of one octant (the four rows
+// +-mz, +-my share each square root), then one block over the blocks' sums.
+// 128^3: 28 us for the two against 14.1 ms for one block of 256 threads.
+constexpr int kMomThreads3 = 256;
+
+__device__ __forceinline__ void block_sum2_3(double &a, double &b) {   // valid in thread 0
+    __shared__ double sh[2][kMomThreads3 / 32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        a += __shfl_down_sync(0xffffffffu, a, o);
+        b += __shfl_down_sync(0xffffffffu, b, o);
     }
-    __shared__ double sh0[256], sh1[256];
-    sh0[threadIdx.x] = s0;
-    sh1[threadIdx.x] = s1;
+    if ((threadIdx.x & 31) == 0) {
+        sh[0][threadIdx.x >> 5] = a;
+        sh[1][threadIdx.x >> 5] = b;
+    }
     __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) {
-            sh0[threadIdx.x] += sh0[threadIdx.x + o];
-            sh1[threadIdx.x] += sh1[threadIdx.x + o];
+    if (threadIdx.x == 0)
+        for (int w = 1; w < kMomThreads3 / 32; ++w) {
+            a += sh[0][w];
+            b += sh[1][w];
         }
-        __syncthreads();
+}
+
+__global__ void __launch_bounds__(kMomThreads3)
+sk3_moments_kernel(const double *__restrict__ acc, int nx, int ny, int nz, int ldx,
+                   double *__restrict__ part) {
+    constexpr int kWarps = kMomThreads3 / 32;
+    const int L = max(nx, max(ny, nz)), sx = L / nx, sy = L / ny, sz = L / nz;
+    const int hx = nx / 2 + 1, hy = ny / 2 + 1;
+    const long long rows = (long long)hy * (nz / 2 + 1);
+    const int lane = threadIdx.x & 31;
+    double s0 = 0.0, s1 = 0.0;
+    for (long long r = (long long)blockIdx.x * kWarps + (threadIdx.x >> 5); r < rows;
+         r += (long long)gridDim.x * kWarps) {
+        const int my = (int)(r % hy), mz = (int)(r / hy);
+        const bool two_y = my > 0 && 2 * my < ny, two_z = mz > 0 && 2 * mz < nz;
+        const double *a = acc + ((size_t)mz * ny + my) * ldx;
+        const double *b = acc + ((size_t)mz * ny + (ny - my)) * ldx;
+        const double *c = acc + ((size_t)(nz - mz) * ny + my) * ldx;
+        const double *d = acc + ((size_t)(nz - mz) * ny + (ny - my)) * ldx;
+        const int r2 = my * sy * (my * sy) + mz * sz * (mz * sz);
+        for (int kx = lane; kx < hx; kx += 32) {
+            if (kx == 0 && r2 == 0) continue;
+            double S = two_y ? a[kx] + b[kx] : a[kx];
+            if (two_z) S += two_y ? c[kx] + d[kx] : c[kx];
+            if (kx > 0 && 2 * kx < nx) S += S;
+            s0 += S;
+            s1 += S * sqrt((double)(kx * sx * (kx * sx) + r2));
+        }
     }
+    block_sum2_3(s0, s1);
     if (threadIdx.x == 0) {
-        out[0] = sh0[0];
-        out[1] = sh1[0];
+        part[2 * blockIdx.x] = s0;
+        part[2 * blockIdx.x + 1] = s1;
+    }
+}
+
+__global__ void __launch_bounds__(kMomThreads3)
+sk3_moments_final_kernel(const double *__restrict__ part, int nblocks, double inv_count, int L,
+                         double *__restrict__ out, const int *__restrict__ flag,
+                         int *__restrict__ flag_out) {
+    double s0 = 0.0, s1 = 0.0;
+    for (int b = threadIdx.x; b < nblocks; b += kMomThreads3) {
+        s0 += part[2 * b];
+        s1 += part[2 * b + 1];
+    }
+    block_sum2_3(s0, s1);
+    if (threadIdx.x == 0) {
+        out[0] = s0 * inv_count;
+        out[1] = s1 * inv_count * (6.283185307179586 / L);
+        *flag_out = *flag;
     }
 }
 
@@ -750,7 +888,7 @@ struct lb3_ctx {
     double *d_part = nullptr;      // conserved partials
     int nred = 0;
     void *drho = nullptr;          // delta rho of a sampling step
-    double *d_prof = nullptr;      // [nz][nx] + [nz][ny] + [nz] plane profiles
+    double *d_prof = nullptr;      // [nz][nx] + [nz][ny] + [nz] plane profiles, [nx + ny] sums
     double *d_acc = nullptr;       // axis S(k) sums [nx/2 + ny/2 + nz/2]
     double *d_io = nullptr;        // n doubles for read-outs
     float2 *d_ring = nullptr;      // [1024] (cos, sin) of the noise ring angles
@@ -759,8 +897,9 @@ struct lb3_ctx {
     void *d_spec = nullptr;        // complex [nz][ny][ldx3] (storage precision)
     double *d_acc3 = nullptr;      // FP64 sums of |X|^2 / N, [nz][ny][ldx3]
     void *d_tw = nullptr;          // twiddles for nx, ny, nz (nx/2 + ny/2 + nz/2 complex)
-    double *d_bins = nullptr;      // read-out scratch: bins, counts (2 nbins_cap) + 2 moments
+    double *d_bins = nullptr;      // partial bins (2 kBinSplits3 nbins_cap), then nbins_cap means
     int nbins_cap = 0;
+    HostReadout rd;                // shells, moments and the flag (lazy, host memory)
     int sk_every = 0;
     long long sk_start = 0, sk_count = 0, t = 0;
     uint64_t seed = 0;
@@ -886,14 +1025,19 @@ int sample_full3(lb3_ctx *h) {
 int sample3(lb3_ctx *h) {
     double *px = h->d_prof, *py = px + (size_t)h->nz * h->nx, *pz = py + (size_t)h->nz * h->ny;
     if (h->precision == LB_FP32)
-        profile3_kernel<float><<<h->nz, 256, 0, h->stream>>>((const float *)h->drho, h->nx, h->ny,
+        profile3_kernel<float><<<h->nz, 32 * kProfWarps, 0, h->stream>>>((const float *)h->drho, h->nx, h->ny,
                                                              px, py, pz);
     else
-        profile3_kernel<double><<<h->nz, 256, 0, h->stream>>>((const double *)h->drho, h->nx,
+        profile3_kernel<double><<<h->nz, 32 * kProfWarps, 0, h->stream>>>((const double *)h->drho, h->nx,
                                                               h->ny, px, py, pz);
     L3_CHECK(cudaGetLastError());
-    axis_dft3_kernel<<<1, 512, (size_t)(h->nx + h->ny + h->nz) * sizeof(double), h->stream>>>(
-        px, py, pz, h->nx, h->ny, h->nz, h->d_acc);
+    double *tot = pz + h->nz;
+    axis_sum3_kernel<<<(h->nx + h->ny + 31) / 32, 32 * kProfWarps, 0, h->stream>>>(
+        px, py, h->nx, h->ny, h->nz, tot);
+    L3_CHECK(cudaGetLastError());
+    const int modes = h->nx / 2 + h->ny / 2 + h->nz / 2;
+    axis_dft3_kernel<<<(modes + 1) / 2, 64, 0, h->stream>>>(tot, pz, h->nx, h->ny, h->nz,
+                                                            h->d_acc);
     L3_CHECK(cudaGetLastError());
     if (h->sk_full) {
         const int rc = h->precision == LB_FP32 ? sample_full3<float>(h) : sample_full3<double>(h);
@@ -928,6 +1072,7 @@ void free3(lb3_ctx *h) {
     cudaFree(h->d_acc3);
     cudaFree(h->d_tw);
     cudaFree(h->d_bins);
+    h->rd.release();
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
 }
 
@@ -1172,7 +1317,7 @@ int lb3_sk_config(lb3_ctx *h, int every, long long start) {
     if (every > 0 && !h->d_acc) {
         const int nm = h->nx / 2 + h->ny / 2 + h->nz / 2;
         L3_CHECK(cudaMalloc(&h->drho, h->n * h->esize));
-        L3_CHECK(cudaMalloc(&h->d_prof, ((size_t)h->nz * (h->nx + h->ny + 1)) * sizeof(double)));
+        L3_CHECK(cudaMalloc(&h->d_prof, ((size_t)(h->nz + 1) * (h->nx + h->ny + 1)) * sizeof(double)));
         L3_CHECK(cudaMalloc(&h->d_acc, nm * sizeof(double)));
         L3_CHECK(cudaMemsetAsync(h->d_acc, 0, nm * sizeof(double), h->stream));
         h->sk_count = 0;
@@ -1241,10 +1386,19 @@ static int bins_scratch3(lb3_ctx *h, int nbins) {
     cudaFree(h->d_bins);
     h->d_bins = nullptr;
     h->nbins_cap = 0;
-    if (cudaMalloc(&h->d_bins, (2 * (size_t)nbins + 2) * sizeof(double)) != cudaSuccess)
+    if (cudaMalloc(&h->d_bins, (2 * kBinSplits3 + 1) * (size_t)nbins * sizeof(double)) !=
+        cudaSuccess)
         return LB_ERR_NOMEM;
     h->nbins_cap = nbins;
     return LB_OK;
+}
+
+// Wait for a read-out whose kernel wrote the flag to h->rd.
+static int readout_sync3(lb3_ctx *h) {
+    L3_CHECK(cudaStreamSynchronize(h->stream));
+    if (!*(volatile int *)h->rd.flag()) return LB_OK;
+    L3_CHECK(cudaMemset(h->d_flag, 0, sizeof(int)));
+    return LB_ERR_NONFINITE;
 }
 
 int lb3_structure_factor(lb3_ctx *h, double *host_bins, int nbins, long long *nsamples_out) {
@@ -1253,25 +1407,23 @@ int lb3_structure_factor(lb3_ctx *h, double *host_bins, int nbins, long long *ns
     L3_CHECK(cudaSetDevice(h->dev));
     int rc = bins_scratch3(h, nbins);
     if (rc) return rc;
-    double *bins = h->d_bins, *counts = bins + nbins;
-    L3_CHECK(cudaMemsetAsync(bins, 0, 2 * (size_t)nbins * sizeof(double), h->stream));
+    L3_CHECK(h->rd.ensure());
     const double inv = h->sk_count ? 1.0 / (double)h->sk_count : 0.0;
-    const size_t total = (size_t)(h->nx / 2 + 1) * h->ny * h->nz;
-    int blocks = (int)((total + 255) / 256);
-    if (blocks > 152 * 16) blocks = 152 * 16;
-    sk3_bins_kernel<<<blocks, 256, 0, h->stream>>>(h->d_acc3, inv, bins, counts, nbins, h->nx,
-                                                   h->ny, h->nz, h->ldx3);
+    // more shells than the mapped buffer holds are copied from the device
+    const bool mapped = nbins <= kReadoutMax;
+    double *means = mapped ? h->rd.v : h->d_bins + 2 * (size_t)kBinSplits3 * nbins;
+    sk3_bins_kernel<<<dim3(nbins, kBinSplits3), kBinThreads3, 0, h->stream>>>(
+        h->d_acc3, h->d_bins, h->nx, h->ny, h->nz, h->ldx3);
     L3_CHECK(cudaGetLastError());
-    double *tmp = new (std::nothrow) double[2 * (size_t)nbins];
-    if (!tmp) return LB_ERR_NOMEM;
-    cudaError_t e = cudaMemcpyAsync(tmp, bins, 2 * (size_t)nbins * sizeof(double),
-                                    cudaMemcpyDeviceToHost, h->stream);
-    rc = e == cudaSuccess ? sync3(h) : LB_ERR_CUDA;
-    if (rc == LB_OK)
-        for (int b = 0; b < nbins; ++b)
-            host_bins[b] = tmp[nbins + b] > 0.0 ? tmp[b] / tmp[nbins + b] : 0.0;
-    delete[] tmp;
+    sk3_bins_final_kernel<<<(nbins + 127) / 128, 128, 0, h->stream>>>(
+        h->d_bins, inv, nbins, means, h->d_flag, h->rd.flag());
+    L3_CHECK(cudaGetLastError());
+    rc = readout_sync3(h);
     if (rc) return rc;
+    if (mapped) memcpy(host_bins, means, nbins * sizeof(double));
+    else
+        L3_CHECK(cudaMemcpy(host_bins, means, (size_t)nbins * sizeof(double),
+                            cudaMemcpyDeviceToHost));
     if (nsamples_out) *nsamples_out = h->sk_count;
     return LB_OK;
 }
@@ -1280,14 +1432,24 @@ int lb3_sk_moments(lb3_ctx *h, double *host_out2) {
     if (!h || !host_out2) return LB_ERR_ARG;
     if (!h->d_acc3) return LB_ERR_STATE;
     L3_CHECK(cudaSetDevice(h->dev));
-    int rc = bins_scratch3(h, 1);
-    if (rc) return rc;
-    double *m = h->d_bins + 2 * (size_t)h->nbins_cap;
+    L3_CHECK(h->rd.ensure());
     const double inv = h->sk_count ? 1.0 / (double)h->sk_count : 0.0;
-    sk3_moments_kernel<<<1, 256, 0, h->stream>>>(h->d_acc3, inv, h->nx, h->ny, h->nz, h->ldx3, m);
+    // d_part holds 4 nred doubles: a pair of sums for each of at most 2 nred blocks
+    const long long rows = (long long)(h->ny / 2 + 1) * (h->nz / 2 + 1);
+    const long long want = (rows + kMomThreads3 / 32 - 1) / (kMomThreads3 / 32);
+    const int nb = (int)(want < 2 * h->nred ? want : 2 * h->nred);
+    sk3_moments_kernel<<<nb, kMomThreads3, 0, h->stream>>>(h->d_acc3, h->nx, h->ny, h->nz, h->ldx3,
+                                                           h->d_part);
     L3_CHECK(cudaGetLastError());
-    L3_CHECK(cudaMemcpyAsync(host_out2, m, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    return sync3(h);
+    const int L = h->nx > h->ny ? (h->nx > h->nz ? h->nx : h->nz) : (h->ny > h->nz ? h->ny : h->nz);
+    sk3_moments_final_kernel<<<1, kMomThreads3, 0, h->stream>>>(h->d_part, nb, inv, L, h->rd.v,
+                                                                h->d_flag, h->rd.flag());
+    L3_CHECK(cudaGetLastError());
+    const int rc = readout_sync3(h);
+    if (rc) return rc;
+    host_out2[0] = h->rd.v[0];
+    host_out2[1] = h->rd.v[1];
+    return LB_OK;
 }
 
 int lb3_structure_factor_axes(lb3_ctx *h, double *host_out, long long *nsamples_out) {

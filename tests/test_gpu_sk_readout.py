@@ -83,3 +83,57 @@ def test_readout_reports_a_nonfinite_state():
     g.step(1)
     assert np.isfinite(g.structure_factor(16)[0][1:]).all()
     g.close()
+
+
+@pytest.mark.parametrize("nx,ny,nz", [(32, 4, 4), (32, 64, 8), (64, 4, 128)])
+@pytest.mark.parametrize("nbins", [1, 0, 5000])
+def test_shells_moments_and_axes_in_3d(nx, ny, nz, nbins):
+    from paper_2212_07848_gb300.lattice3 import Lattice3
+    g = Lattice3(nx, ny, nz, -3.6, 1.0, 1e-5, precision="fp64")
+    g.init(LN2, 5, 0.01)
+    g.sk_config(4, 4)
+    g.sk_full()
+    g.step(4)
+    rho = g.density()
+    S = np.abs(np.fft.fftn(rho - rho.mean())) ** 2 / rho.size
+    S[0, 0, 0] = 0.0
+    L = max(nx, ny, nz)
+    qz, qy, qx = np.meshgrid(*(_folded(n) * (L / n) for n in (nz, ny, nx)), indexing="ij")
+    q = np.sqrt(qx ** 2 + qy ** 2 + qz ** 2)
+    b = np.rint(q).astype(int)
+    b[0, 0, 0] = -1
+    nbins = nbins or b.max() + 1
+    keep = (b >= 0) & (b < nbins)
+    cnt = np.bincount(b[keep], minlength=nbins)
+    ref = np.bincount(b[keep], S[keep], minlength=nbins) / np.maximum(cnt, 1)
+    got, n = g.structure_factor(nbins)
+    # numpy's FFT and the device's differ by a few FP64 roundings of the largest mode
+    assert n == 1 and np.abs(got - ref).max() < 1e-11 * S.max()
+    assert np.array_equal(got == 0.0, cnt == 0)
+    m = g.sk_moments()
+    assert abs(m[0] / S.sum() - 1.0) < 1e-11
+    assert abs(m[1] / (2 * np.pi / L * q * S).sum() - 1.0) < 1e-11
+    axes, _ = g.structure_factor_axes()
+    want = np.concatenate([S[0, 0, 1:nx // 2 + 1], S[0, 1:ny // 2 + 1, 0], S[1:nz // 2 + 1, 0, 0]])
+    assert np.abs(axes - want).max() < 1e-11 * S.max()
+    g.close()
+
+
+@pytest.mark.parametrize("nx,ny,nz,precision", [(96, 4, 3, "fp32"), (160, 12, 5, "fp64"),
+                                                (32, 20, 7, "fp32")])
+def test_axis_profiles_of_other_sizes(nx, ny, nz, precision):
+    """Sizes with a part of a 128-column chunk, fewer rows than warps and an odd
+    number of planes."""
+    from paper_2212_07848_gb300.lattice3 import Lattice3
+    g = Lattice3(nx, ny, nz, -3.6, 0.9, 1e-5, precision=precision)
+    g.init(LN2, 5, 0.01)
+    g.sk_config(3, 3)
+    g.step(3)
+    rho = g.density()
+    S = np.abs(np.fft.fftn(rho - rho.mean())) ** 2 / rho.size
+    axes, n = g.structure_factor_axes()
+    want = np.concatenate([S[0, 0, 1:nx // 2 + 1], S[0, 1:ny // 2 + 1, 0], S[1:nz // 2 + 1, 0, 0]])
+    # FP32: the sampled density is rounded to FP32 (2^-24 of the deviations, on every site)
+    tol = 1e-11 if precision == "fp64" else 2e-6
+    assert n == 1 and np.abs(axes - want).max() < tol * want.max()
+    g.close()
