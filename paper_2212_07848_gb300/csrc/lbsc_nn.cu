@@ -280,13 +280,24 @@ wgrad_kernel(const bf16 *__restrict__ x, const bf16 *__restrict__ dy, float *__r
             }
 }
 
-// dw[i] += sum over chunks of part[chunk][i], chunks added in order.
-__global__ void wgrad_reduce_kernel(const float *__restrict__ part, float *__restrict__ dw, size_t n,
-                                    int nchunk) {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
-         i += (size_t)gridDim.x * blockDim.x) {
-        float s = 0.f;
-        for (int ch = 0; ch < nchunk; ++ch) s += part[(size_t)ch * n + i];
+// dw[i] += sum over chunks of part[chunk][i]: 32 weights to a block, its eight
+// warps sum every eighth chunk and are added in order (a fixed order).  Bound by
+// the partial sums' bytes where there are many weights (64 -> 128: 83 MB, 10.9 us,
+// 13.9 before) and by the chain of loads where there are few: one thread per weight
+// over all chunks left 18 blocks for 16 -> 32 (33.6 us; 8.6 us now).
+constexpr int kRedWarps = 8;
+__global__ void __launch_bounds__(32 * kRedWarps)
+wgrad_reduce_kernel(const float *__restrict__ part, float *__restrict__ dw, size_t n, int nchunk) {
+    __shared__ float sh[kRedWarps][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const size_t i = (size_t)blockIdx.x * 32 + lane;   // n is a multiple of 32
+    float s = 0.f;
+#pragma unroll 8
+    for (int ch = w; ch < nchunk; ch += kRedWarps) s += part[(size_t)ch * n + i];
+    sh[w][lane] = s;
+    __syncthreads();
+    if (w == 0) {
+        for (int k = 1; k < kRedWarps; ++k) s += sh[k][lane];
         dw[i] += s;
     }
 }
@@ -380,9 +391,55 @@ __global__ void __launch_bounds__(256) bias_reduce_kernel(const float *__restric
     if (threadIdx.x == 0) db[c] += red[0];
 }
 
+// The elementwise passes are bound by memory traffic.  Where the channel count is
+// a multiple of 8 and the buffers are 16-byte aligned (every layer of the
+// surrogate) a thread moves eight channels with 16-byte accesses, and the pooling
+// and upsampling kernels walk whole rows, so that a thread's channel group costs
+// one 32-bit remainder instead of a 64-bit division per element.  Other shapes
+// take the kernels with one element per thread.  8 x 512^2 training iteration
+// (us, one element per thread -> now): up2 917 -> 99, its gradient 267 -> 73, pool2
+// 139 -> 49, its gradient 474 -> 78, relu mask 504 -> 129, add 134 -> 57.
+struct alignas(16) Bf8 {
+    __nv_bfloat162 e[4];
+};
+__device__ __forceinline__ Bf8 ld8(const bf16 *p) { return *reinterpret_cast<const Bf8 *>(p); }
+__device__ __forceinline__ void st8(bf16 *p, const Bf8 &v) { *reinterpret_cast<Bf8 *>(p) = v; }
+__device__ __forceinline__ void to_f8(const Bf8 &v, float f[8]) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float2 t = __bfloat1622float2(v.e[k]);
+        f[2 * k] = t.x;
+        f[2 * k + 1] = t.y;
+    }
+}
+__device__ __forceinline__ Bf8 from_f8(const float f[8]) {
+    Bf8 v;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v.e[k] = __floats2bfloat162_rn(f[2 * k], f[2 * k + 1]);
+    return v;
+}
+inline bool aligned16(const void *a, const void *b, const void *c = nullptr) {
+    return (((uintptr_t)a | (uintptr_t)b | (uintptr_t)c) & 15) == 0;
+}
+
 __global__ void relu_mask_kernel(const bf16 *__restrict__ dy, const bf16 *__restrict__ y,
                                  bf16 *__restrict__ dz, size_t n) {
     GRID_STRIDE(i, n) dz[i] = __bfloat162float(y[i]) > 0.f ? dy[i] : __float2bfloat16(0.f);
+}
+__device__ __forceinline__ Bf8 mask8(const Bf8 &d, const Bf8 &y) {
+    Bf8 r;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float2 t = __bfloat1622float2(y.e[k]);
+        r.e[k].x = t.x > 0.f ? d.e[k].x : __float2bfloat16(0.f);
+        r.e[k].y = t.y > 0.f ? d.e[k].y : __float2bfloat16(0.f);
+    }
+    return r;
+}
+__global__ void __launch_bounds__(256)
+relu_mask8_kernel(const bf16 *__restrict__ dy, const bf16 *__restrict__ y, bf16 *__restrict__ dz,
+                  size_t n8) {
+    GRID_STRIDE(i, n8) st8(dz + 8 * i, mask8(ld8(dy + 8 * i), ld8(y + 8 * i)));
 }
 
 __global__ void pool2_fwd_kernel(const bf16 *__restrict__ x, bf16 *__restrict__ y, int NB, int H,
@@ -438,9 +495,78 @@ __global__ void up2_bwd_kernel(const bf16 *__restrict__ dy, bf16 *__restrict__ d
     }
 }
 
+// Between images [rows][w][C] and [2 rows][2 w][C] (rows = images x coarse
+// height), eight channels per thread: COARSEN adds the four fine pixels of a
+// coarse one and scales the sum, else a coarse pixel is scaled and written to
+// its four.  Pooling is <true> with scale 1/4 and its gradient <false> with 1/4;
+// upsampling is <false> with 1 and its gradient <true> with 1 (scaling by these
+// is exact).
+template <bool COARSEN>
+__global__ void __launch_bounds__(256)
+quad8_kernel(const bf16 *__restrict__ in, bf16 *__restrict__ out, unsigned rows, unsigned w,
+             unsigned C, float scale) {
+    const unsigned G = C / 8, wg = w * G, row_f = 2 * w * C;   // fine row, in values
+    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= wg) return;
+    const unsigned g = i % G;
+    const unsigned fine = 16 * (i - g) + 8 * g;   // (2 x) C + 8 g with x = (i - g) / G
+    for (size_t r = blockIdx.y; r < rows; r += gridDim.y) {
+        const size_t c0 = r * w * C + 8 * (size_t)i, f0 = 2 * r * row_f + fine;
+        float a[8];
+        if (COARSEN) {
+            float q[3][8];
+            to_f8(ld8(in + f0), a);
+            to_f8(ld8(in + f0 + C), q[0]);
+            to_f8(ld8(in + f0 + row_f), q[1]);
+            to_f8(ld8(in + f0 + row_f + C), q[2]);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) a[k] = scale * (((a[k] + q[0][k]) + q[1][k]) + q[2][k]);
+            st8(out + c0, from_f8(a));
+        } else {
+            Bf8 v = ld8(in + c0);
+            if (scale != 1.f) {
+                to_f8(v, a);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) a[k] *= scale;
+                v = from_f8(a);
+            }
+            st8(out + f0, v);
+            st8(out + f0 + C, v);
+            st8(out + f0 + row_f, v);
+            st8(out + f0 + row_f + C, v);
+        }
+    }
+}
+
+// The 8-channel kernel where it applies; false: the caller takes the general one.
+template <bool COARSEN>
+bool launch_quad8(const void *in, void *out, int nb, int hc, int wc, int C, float scale,
+                  cudaStream_t s) {
+    if (nb < 1 || hc < 1 || wc < 1 || C < 8 || C % 8 || !aligned16(in, out)) return false;
+    const size_t rows = (size_t)nb * hc, wg = (size_t)wc * (C / 8);
+    if (rows >= (1ull << 32) || (size_t)wc * C >= (1ull << 30)) return false;
+    const dim3 grid((unsigned)((wg + 255) / 256), (unsigned)(rows < 65535 ? rows : 65535));
+    quad8_kernel<COARSEN><<<grid, 256, 0, s>>>((const bf16 *)in, (bf16 *)out, (unsigned)rows,
+                                               (unsigned)wc, (unsigned)C, scale);
+    return true;
+}
+
 __global__ void add_kernel(const bf16 *__restrict__ a, const bf16 *__restrict__ b,
                            bf16 *__restrict__ y, size_t n) {
     GRID_STRIDE(i, n) y[i] = __float2bfloat16(__bfloat162float(a[i]) + __bfloat162float(b[i]));
+}
+__device__ __forceinline__ Bf8 add8(const Bf8 &a, const Bf8 &b) {
+    float fa[8], fb[8];
+    to_f8(a, fa);
+    to_f8(b, fb);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) fa[k] += fb[k];
+    return from_f8(fa);
+}
+__global__ void __launch_bounds__(256)
+add8_kernel(const bf16 *__restrict__ a, const bf16 *__restrict__ b, bf16 *__restrict__ y,
+            size_t n8) {
+    GRID_STRIDE(i, n8) st8(y + 8 * i, add8(ld8(a + 8 * i), ld8(b + 8 * i)));
 }
 
 // Coarse-grain the density of a lattice state (FP32 deviations [9][ny][nx])
@@ -568,20 +694,42 @@ __global__ void mse_ch_kernel(const bf16 *__restrict__ y, int C, int ch,
 
 // Residual MSE: prediction = base + y[.][0] (FP32 base, BF16 increment),
 // loss += mean((prediction - target)^2), dy = d loss / d y (channel 0; 0 elsewhere).
-__global__ void mse_kernel(const bf16 *__restrict__ y, int C, const float *__restrict__ tgt,
-                           const float *__restrict__ base, size_t n, float *__restrict__ loss,
-                           bf16 *__restrict__ dy) {
+// VEC (C a multiple of 8, dy 16-byte aligned): a pixel's channels leave as 16-byte
+// stores.  One atomic per block.  8 x 512^2, 16 channels: 47 us against
+// 174 us with 2-byte stores and an atomic per warp; bound by dy's bytes.
+template <bool VEC>
+__global__ void __launch_bounds__(256)
+mse_kernel(const bf16 *__restrict__ y, int C, const float *__restrict__ tgt,
+           const float *__restrict__ base, size_t n, float *__restrict__ loss,
+           bf16 *__restrict__ dy) {
     float s = 0.f;
     GRID_STRIDE(i, n) {
         const float d = base[i] + __bfloat162float(y[i * C]) - tgt[i];
         s += d * d;
         if (dy) {
-            dy[i * C] = __float2bfloat16(2.f * d / (float)n);
-            for (int c = 1; c < C; ++c) dy[i * C + c] = __float2bfloat16(0.f);
+            const float g = 2.f * d / (float)n;
+            if (VEC) {
+                Bf8 v;
+                const __nv_bfloat162 z = __floats2bfloat162_rn(0.f, 0.f);
+                v.e[0] = __floats2bfloat162_rn(g, 0.f);
+                v.e[1] = v.e[2] = v.e[3] = z;
+                st8(dy + i * C, v);
+                v.e[0] = z;
+                for (int c = 8; c < C; c += 8) st8(dy + i * C + c, v);
+            } else {
+                dy[i * C] = __float2bfloat16(g);
+                for (int c = 1; c < C; ++c) dy[i * C + c] = __float2bfloat16(0.f);
+            }
         }
     }
+    __shared__ float red[8];
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(loss, s / (float)n);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) s += red[w];
+        atomicAdd(loss, s / (float)n);
+    }
 }
 
 // Mean of channel 0 of y [n][C] in two passes with a fixed summation order:
@@ -649,11 +797,23 @@ __global__ void adam_kernel(float *__restrict__ w, const float *__restrict__ g, 
 
 // Network input from an FP32 field: out[i][0] = BF16(src[i]), out[i][1] = gfeat,
 // out[i][2] = BF16(src[i] - prev[i]) (the last increment; 0 without prev),
-// out[i][3..C) = 0.
+// out[i][3..C) = 0.  VEC (C a multiple of 8, out 16-byte aligned): 16-byte stores.
+template <bool VEC>
 __global__ void expand_kernel(const float *__restrict__ src, const float *__restrict__ prev,
                               float gfeat, bf16 *__restrict__ out, int C, size_t n) {
     GRID_STRIDE(i, n) {
         bf16 *o = out + i * C;
+        if (VEC) {
+            Bf8 v;
+            const __nv_bfloat162 z = __floats2bfloat162_rn(0.f, 0.f);
+            v.e[0] = __floats2bfloat162_rn(src[i], gfeat);
+            v.e[1] = __floats2bfloat162_rn(prev ? src[i] - prev[i] : 0.f, 0.f);
+            v.e[2] = v.e[3] = z;
+            st8(o, v);
+            v.e[0] = v.e[1] = z;
+            for (int c = 8; c < C; c += 8) st8(o + c, v);
+            continue;
+        }
         o[0] = __float2bfloat16(src[i]);
         if (C > 1) o[1] = __float2bfloat16(gfeat);
         if (C > 2) o[2] = __float2bfloat16(prev ? src[i] - prev[i] : 0.f);
@@ -814,7 +974,7 @@ int lb_nn_conv3x3_wgrad(const void *x, const void *dy, float *dw, float *dbias, 
         if (cudaGetLastError() != cudaSuccess) return LB_ERR_CUDA;
         nchunk = p.nchunk;
     }
-    wgrad_reduce_kernel<<<blocks_for(n), 256, 0, s>>>(part, dw, n, nchunk);
+    wgrad_reduce_kernel<<<(unsigned)(n / 32), 32 * kRedWarps, 0, s>>>(part, dw, n, nchunk);
     if (cudaGetLastError() != cudaSuccess) return LB_ERR_CUDA;
     if (dbias) {
         bias_grad_kernel<<<kBiasBlocks, 256, 0, s>>>(db, bpart, (size_t)nb * h * wd, cout);
@@ -825,33 +985,50 @@ int lb_nn_conv3x3_wgrad(const void *x, const void *dy, float *dw, float *dbias, 
 }
 
 int lb_nn_relu_mask(const void *dy, const void *y, void *dz, size_t n, void *stream) {
-    relu_mask_kernel<<<blocks_for(n), 256, 0, (cudaStream_t)stream>>>(
-        (const bf16 *)dy, (const bf16 *)y, (bf16 *)dz, n);
+    if (n % 8 == 0 && aligned16(dy, y, dz))
+        relu_mask8_kernel<<<blocks_for(n / 8), 256, 0, (cudaStream_t)stream>>>(
+            (const bf16 *)dy, (const bf16 *)y, (bf16 *)dz, n / 8);
+    else
+        relu_mask_kernel<<<blocks_for(n), 256, 0, (cudaStream_t)stream>>>(
+            (const bf16 *)dy, (const bf16 *)y, (bf16 *)dz, n);
     NN_RET();
 }
 
 int lb_nn_pool2(const void *x, void *y, int nb, int h, int w, int c, int backward, void *stream) {
     if (h % 2 || w % 2) return LB_ERR_ARG;
     const size_t n = backward ? (size_t)nb * h * w * c : (size_t)nb * (h / 2) * (w / 2) * c;
+    cudaStream_t s = (cudaStream_t)stream;
+    if (backward ? launch_quad8<false>(x, y, nb, h / 2, w / 2, c, 0.25f, s)
+                 : launch_quad8<true>(x, y, nb, h / 2, w / 2, c, 0.25f, s))
+        NN_RET();
     if (!backward)
-        pool2_fwd_kernel<<<blocks_for(n), 256, 0, (cudaStream_t)stream>>>((const bf16 *)x, (bf16 *)y, nb, h, w, c);
+        pool2_fwd_kernel<<<blocks_for(n), 256, 0, s>>>((const bf16 *)x, (bf16 *)y, nb, h, w, c);
     else
-        pool2_bwd_kernel<<<blocks_for(n), 256, 0, (cudaStream_t)stream>>>((const bf16 *)x, (bf16 *)y, nb, h, w, c);
+        pool2_bwd_kernel<<<blocks_for(n), 256, 0, s>>>((const bf16 *)x, (bf16 *)y, nb, h, w, c);
     NN_RET();
 }
 
 int lb_nn_up2(const void *x, void *y, int nb, int h, int w, int c, int backward, void *stream) {
     // (h, w): the coarse size
     const size_t n = backward ? (size_t)nb * h * w * c : (size_t)nb * 4 * h * w * c;
+    cudaStream_t s = (cudaStream_t)stream;
+    if (backward ? launch_quad8<true>(x, y, nb, h, w, c, 1.f, s)
+                 : launch_quad8<false>(x, y, nb, h, w, c, 1.f, s))
+        NN_RET();
     if (!backward)
-        up2_fwd_kernel<<<blocks_for(n), 256, 0, (cudaStream_t)stream>>>((const bf16 *)x, (bf16 *)y, nb, h, w, c);
+        up2_fwd_kernel<<<blocks_for(n), 256, 0, s>>>((const bf16 *)x, (bf16 *)y, nb, h, w, c);
     else
-        up2_bwd_kernel<<<blocks_for(n), 256, 0, (cudaStream_t)stream>>>((const bf16 *)x, (bf16 *)y, nb, h, w, c);
+        up2_bwd_kernel<<<blocks_for(n), 256, 0, s>>>((const bf16 *)x, (bf16 *)y, nb, h, w, c);
     NN_RET();
 }
 
 int lb_nn_add(const void *a, const void *b, void *y, size_t n, void *stream) {
-    add_kernel<<<blocks_for(n), 256, 0, (cudaStream_t)stream>>>((const bf16 *)a, (const bf16 *)b, (bf16 *)y, n);
+    if (n % 8 == 0 && aligned16(a, b, y))
+        add8_kernel<<<blocks_for(n / 8), 256, 0, (cudaStream_t)stream>>>(
+            (const bf16 *)a, (const bf16 *)b, (bf16 *)y, n / 8);
+    else
+        add_kernel<<<blocks_for(n), 256, 0, (cudaStream_t)stream>>>((const bf16 *)a, (const bf16 *)b,
+                                                                    (bf16 *)y, n);
     NN_RET();
 }
 
@@ -910,8 +1087,12 @@ int lb_nn_mse_channel(const void *y, int c, int ch, const float *target, const f
 int lb_nn_mse(const void *y, int c, const float *target, const float *base, size_t n, float *loss,
               void *dy, void *stream) {
     if (!y || !target || !base || !loss || c < 1) return LB_ERR_ARG;
-    mse_kernel<<<blocks_for(n), 256, 0, (cudaStream_t)stream>>>(
-        (const bf16 *)y, c, target, base, n, loss, (bf16 *)dy);
+    if (dy && c % 8 == 0 && aligned16(dy, nullptr))
+        mse_kernel<true><<<blocks_for(n), 256, 0, (cudaStream_t)stream>>>(
+            (const bf16 *)y, c, target, base, n, loss, (bf16 *)dy);
+    else
+        mse_kernel<false><<<blocks_for(n), 256, 0, (cudaStream_t)stream>>>(
+            (const bf16 *)y, c, target, base, n, loss, (bf16 *)dy);
     NN_RET();
 }
 
@@ -943,8 +1124,12 @@ int lb_nn_adam(float *w, const float *g, float *m, float *v, void *w_bf16, size_
 int lb_nn_expand(const float *src, const float *prev, double gfeat, void *out, int c, size_t n,
                  void *stream) {
     if (!src || !out || c < 1) return LB_ERR_ARG;
-    expand_kernel<<<blocks_for(n), 256, 0, (cudaStream_t)stream>>>(src, prev, (float)gfeat,
-                                                                   (bf16 *)out, c, n);
+    if (c % 8 == 0 && aligned16(out, nullptr))
+        expand_kernel<true><<<blocks_for(n), 256, 0, (cudaStream_t)stream>>>(
+            src, prev, (float)gfeat, (bf16 *)out, c, n);
+    else
+        expand_kernel<false><<<blocks_for(n), 256, 0, (cudaStream_t)stream>>>(
+            src, prev, (float)gfeat, (bf16 *)out, c, n);
     NN_RET();
 }
 
