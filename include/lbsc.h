@@ -70,14 +70,16 @@ extern "C" {
 
 /* ---- step kernel selection (lb_set_kernel) -------------------------------- */
 #define LB_KERNEL_AUTO 0    /* the fastest kernel for this GPU and lattice: on
-                               GB300 overlap for nx >= 1024, else plain          */
-#define LB_KERNEL_PLAIN 1   /* coalesced global loads; strips of 128 columns and a
-                               fifth warp for the halo columns' pseudopotential   */
+                               GB300 overlap for nx >= 1024, else plain, and tiles
+                               instead of strips on smaller lattices              */
+#define LB_KERNEL_PLAIN 1   /* coalesced global loads; strips of up to 128 columns
+                               (64 threads, two columns each), tiles on smaller
+                               lattices unless a strip height was set             */
 #define LB_KERNEL_TMA 2     /* rows staged in shared memory by cp.async.bulk.tensor
                                (FP32 and nx a multiple of 128 only)               */
-#define LB_KERNEL_OVERLAP 3 /* coalesced global loads; strips of 128 - 2H columns
-                               whose halo columns are pulled by the CTA's own
-                               threads (no separate halo warp)                    */
+#define LB_KERNEL_OVERLAP 3 /* coalesced global loads; strips of up to 256 columns
+                               (128 threads, two columns each).  FP64 lattices run
+                               one kernel, in tiles, under PLAIN and OVERLAP      */
 
 /* ---- lb_device_ptr selectors -------------------------------------------- */
 #define LB_PTR_POPULATIONS 0   /* current deviations [9][ny][nx] (T)        */
@@ -136,9 +138,10 @@ int lb_init(lb_ctx *h, double rho0, uint64_t seed, double init_amp);
  * seed).  Default 0. */
 int lb_set_replica(lb_ctx *h, uint32_t replica);
 
-/* Rows of the lattice swept by one CTA of the step kernel (launch-shape
- * tuning, 1 <= rows <= ny; the default depends on the lattice size).  Does
- * not change results. */
+/* Rows of the lattice swept by one CTA of the strip kernels (launch-shape
+ * tuning, 1 <= rows <= ny; the default depends on the lattice size; narrow
+ * lattices sweep several such bands per CTA).  Does not change results, and has
+ * no effect on FP64 lattices, which run in tiles. */
 int lb_set_strip_height(lb_ctx *h, int rows);
 
 /* Choose the step kernel (LB_KERNEL_*).  All kernels perform the same
@@ -333,8 +336,8 @@ int lb_ens_get_launch(const lb_ens *e);
  * ensemble's stream.  Errors: LB_ERR_ARG, LB_ERR_CUDA. */
 int lb_ens_set_wait_ns(lb_ens *e, long long ns);
 /* Strip layout of the ensemble's step kernels, as lb_set_kernel:
- * LB_KERNEL_PLAIN (128-column strips and a halo warp) or LB_KERNEL_OVERLAP
- * (strips of 128 - 2H columns whose halo the CTA's own threads pull);
+ * LB_KERNEL_PLAIN (strips of up to 128 columns) or LB_KERNEL_OVERLAP (of up to
+ * 256);
  * LB_KERNEL_AUTO takes the faster one on this GPU.  Same results either way.
  * Synchronises the ensemble's stream and rebuilds the tile list.
  * lb_ens_get_kernel returns the layout in use.  Errors: LB_ERR_ARG, LB_ERR_CUDA. */

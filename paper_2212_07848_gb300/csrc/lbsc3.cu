@@ -388,7 +388,7 @@ step3_kernel(const K3<T> p) {
             T g[19];
             pull3(p.src, plane, xo, yo, zo, g);
             dnew = sum19(g);
-            s_psi[it & 3][ty][tx] = delta_psi<T>(dnew, p.psi_kind, p.rho0, p.psi_c, p.psi_b);
+            s_psi[it & 3][ty][tx] = delta_psi(dnew, p.psi_kind, p.rho0, p.psi_c, p.psi_b);
             if (UNIT) moments3<T, 4>(g, mnew);
         }
         __syncthreads();

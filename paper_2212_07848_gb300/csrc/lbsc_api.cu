@@ -47,7 +47,7 @@ struct lb_ctx {
     uint64_t seed = 0;
     uint32_t replica = 0;
     long long t = 0;
-    int strip_h = 32;
+    int strip_h = 0;                // rows asked for (lb_set_strip_height), or 0
     int kernel_mode = 0;            // LB_KERNEL_*
     TmaMaps maps;                   // tensor maps of df[0], df[1] (FP32 only)
     long long wait_ns = -1;         // staged kernel's mbarrier bound (< 0: default)
@@ -106,16 +106,12 @@ int validate(const lb_params *p) {
     return LB_ERR_ARG;
 }
 
-int default_strip(int nx, int ny) {
-    const bool ov = nx >= 1024;   // the overlapped kernel (see lb_get_kernel)
-    const long gx = ov ? (nx + kStepTX - 3) / (kStepTX - 2) : (nx + kStepTX - 1) / kStepTX;
-    long target = (long)ny * gx / (152 * 4);
+// Rows per CTA of the staged kernel.
+int tma_strip(int nx, int ny) {
+    const long target = (long)ny * ((nx + 127) / 128) / (152 * 4);
     int h = 8;
     while (h < 32 && h * 2 <= target) h *= 2;
-    // the overlapped kernel measured fastest at 24 rows per CTA (4096^2)
-    if (ov && h == 32) h = 24;
-    if (h > ny) h = ny;
-    return h;
+    return h > ny ? ny : h;
 }
 
 double psi_of(const lb_params &p, double rho) {
@@ -132,7 +128,6 @@ void fill_base(lb_ctx *h) {
     memset(&a, 0, sizeof(a));
     a.nx = p.nx;
     a.ny = p.ny;
-    a.strip_h = h->strip_h;
     a.rho0 = h->rho0;
     a.force_pref = -p.G * kCs2;
     a.psi_kind = p.psi_kind;
@@ -299,7 +294,6 @@ int lb_create_ex(lb_ctx **out, const lb_params *p) {
         delete h;
         return cuda_status(e);
     }
-    h->strip_h = default_strip(p->nx, p->ny);
     if (tma_eligible(p->precision, p->nx, p->ny))
         tma_encode_maps(&h->maps, h->df[0], h->df[1], p->nx, p->ny);
     fill_base(h);
@@ -360,7 +354,6 @@ int lb_set_replica(lb_ctx *h, uint32_t replica) {
 int lb_set_strip_height(lb_ctx *h, int rows) {
     if (!h || rows < 1 || rows > h->p.ny) return LB_ERR_ARG;
     h->strip_h = rows;
-    h->base.strip_h = rows;
     ++h->ver;
     return LB_OK;
 }
@@ -382,12 +375,8 @@ int lb_set_wait_ns(lb_ctx *h, long long ns) {
 
 int lb_get_kernel(const lb_ctx *h) {
     if (!h) return LB_ERR_ARG;
-    // AUTO: on GB300 the overlapped-strip kernel is the fastest for lattices
-    // at least 1024 columns wide (the step is issue-bound; without a halo warp
-    // every resident warp collides, 8 CTAs of 4 warps per SM instead of 6 of
-    // 5: 73 against 67 GLUPS at 4096^2), while narrower lattices lose more to
-    // its partly filled last strip (a power-of-two width leaves a strip of a
-    // few columns) and take the halo-warp kernel.  The staged kernel's per-row
+    // AUTO: strips of 128 threads for lattices at least 1024 columns wide, of 64
+    // for narrower ones (4096^2: 188 against 190 us).  The staged kernel's per-row
     // mbarrier hand-off costs more than the loads it saves.
     if (h->kernel_mode == LB_KERNEL_TMA && h->maps.ok) return LB_KERNEL_TMA;
     if (h->kernel_mode == LB_KERNEL_PLAIN) return LB_KERNEL_PLAIN;
@@ -418,7 +407,14 @@ cudaError_t launch_one(lb_ctx *h, int kern, int buf, bool sample, uint32_t step,
     a.step = step;
     a.clock = clock;
     a.wait_ns = h->wait_ns;
-    a.layout = kern == LB_KERNEL_OVERLAP ? 1 : 0;
+    const bool unit = a.gamma == 0.0 && a.gamma_b == 0.0 && a.gamma_g == 0.0;
+    a.layout = kern == LB_KERNEL_OVERLAP ? kLayoutWide : kLayoutNarrow;
+    if (h->strip_h == 0 && h->kernel_mode != LB_KERNEL_OVERLAP &&
+        tile_is_faster(a.nx, a.ny, unit))
+        a.layout = kLayoutTile;
+    if (h->strip_h > 0) a.strip_h = h->strip_h;
+    else if (kern == LB_KERNEL_TMA) a.strip_h = tma_strip(a.nx, a.ny);
+    else a.strip_h = strip_rows(a.nx, a.ny, a.layout, unit);
     if (kern == LB_KERNEL_TMA) return launch_step_tma(h->p.stencil, a, h->maps, buf, h->stream);
     return launch_step(h->p.precision, h->p.stencil, a, h->stream);
 }

@@ -21,7 +21,8 @@ template <typename T> struct KParams {
     T rho0, force_pref, psi_c, psi_b, psi0;
     T gamma_b, gamma, gamma_g;        // 1 - 1/tau of the bulk, shear and ghost modes
     T c3a, c3b, c4a, c4b, c5a, c5b;   // folded relaxation/source constants
-    T amp[6];
+    T amp[6];                         // minus the noise amplitudes (ring_polar)
+    int unit;                         // every relaxation rate is 1 (see collide)
     uint32_t rk[20];
     // when not null, the step counter of the noise is *clock + step (a
     // captured window of steps replays for any starting step)
@@ -57,16 +58,152 @@ __device__ __forceinline__ void pull(const T *__restrict__ src, size_t plane_, i
     g[8] = ldsrc<CG>(src + (8u * plane + rp + xm));
 }
 
-// 1/rho: FP32 from the reciprocal square root squared; FP64 correctly rounded.
+// 1/rho: FP32 from the reciprocal square root squared (NaN for a negative
+// density, which the step then reports); FP64 correctly rounded.
 __device__ __forceinline__ float inv_rho_of(float rho) {
-    const float r = rsqrtf(rho);
-    return r * r;
+    const float r = hw_rsqrt(rho);
+    return __fmul_rn(r, r);
+}
+__device__ __forceinline__ float2 inv_rho_of(float2 rho) {
+    const float2 r = make_float2(hw_rsqrt(rho.x), hw_rsqrt(rho.y));
+    return vmul(r, r);
 }
 __device__ __forceinline__ double inv_rho_of(double rho) { return 1.0 / rho; }
 
+template <typename V>
+__device__ __forceinline__ V sum9(const V g[9]) {
+    return vadd(vadd(vadd(g[0], vadd(g[1], g[3])), vadd(g[2], g[4])),
+                vadd(vadd(g[5], g[7]), vadd(g[6], g[8])));
+}
+
+// The step counter of the noise for a kernel launched with params p.
 template <typename T>
-__device__ __forceinline__ T sum9(const T g[9]) {
-    return ((g[0] + (g[1] + g[3])) + (g[2] + g[4])) + ((g[5] + g[7]) + (g[6] + g[8]));
+__device__ __forceinline__ uint32_t step_of(const KParams<T> &p) {
+    return p.clock ? p.step + __ldg(p.clock) : p.step;
+}
+
+// Mass and momentum deviations of the pulled populations (the mass in the order of
+// the forward transform, which is not that of sum9).
+template <typename V>
+__device__ __forceinline__ void unit_moments(const V g[9], V &drho, V &m1, V &m2) {
+    const V t1 = vadd(vsub(g[5], g[7]), vsub(g[8], g[6]));
+    const V t2 = vsub(vsub(g[5], g[7]), vsub(g[8], g[6]));
+    drho = vadd(g[0], vadd(vadd(vadd(g[1], g[3]), vadd(g[2], g[4])),
+                           vadd(vadd(g[5], g[7]), vadd(g[6], g[8]))));
+    m1 = vadd(vsub(g[1], g[3]), t1);
+    m2 = vadd(vsub(g[2], g[4]), t2);
+}
+
+// The three ring pairs of a site (or of the sites `site` and `site + 1`): radii
+// with sqrt(rho) folded in, cosines and sines.  One Philox call a site and step:
+// radius words r.x, r.y, r.z and three 10-bit angle indices of r.w.
+template <typename T>
+__device__ __forceinline__ void ring_noise(T rho, const KParams<T> &p,
+                                           const uint32_t *__restrict__ rk, uint32_t site,
+                                           uint32_t step, T rad[3], T c[3], T s[3]) {
+    const uint4 r = philox4x32_10(make_uint4(site, step, p.replica, 0u), rk);
+    ring_polar(uniform01<T>(r.x), r.w & 1023u, rho, rad[0], c[0], s[0]);
+    ring_polar(uniform01<T>(r.y), (r.w >> 10) & 1023u, rho, rad[1], c[1], s[1]);
+    ring_polar(uniform01<T>(r.z), (r.w >> 20) & 1023u, rho, rad[2], c[2], s[2]);
+}
+__device__ __forceinline__ void ring_noise(float2 rho, const KParams<float> &p,
+                                           const uint32_t *__restrict__ rk, uint32_t site,
+                                           uint32_t step, float2 rad[3], float2 c[3],
+                                           float2 s[3]) {
+    const uint4 r0 = philox4x32_10(make_uint4(site, step, p.replica, 0u), rk);
+    const uint4 r1 = philox4x32_10(make_uint4(site + 1u, step, p.replica, 0u), rk);
+    const uint32_t w0[3] = {r0.x, r0.y, r0.z}, w1[3] = {r1.x, r1.y, r1.z};
+    const float2 k = vmul(bc<float2>(-1.3862943611198906f), rho);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const float2 u = vfma(make_float2(__uint2float_rn(w0[j]), __uint2float_rn(w1[j])),
+                              bc<float2>(2.3283064365386963e-10f),
+                              bc<float2>(1.1641532182693481e-10f));
+        const float2 x = vmul(k, make_float2(hw_log2(u.x), hw_log2(u.y)));
+        const float2 h = make_float2(hw_rsqrt(fmaxf(x.x, 1e-30f)), hw_rsqrt(fmaxf(x.y, 1e-30f)));
+        rad[j] = vmul(x, h);
+        const uint32_t a0 = (r0.w >> (10 * j)) & 1023u, a1 = (r1.w >> (10 * j)) & 1023u;
+        const float2 th = vfma(make_float2(__uint2float_rn(a0), __uint2float_rn(a1)),
+                               bc<float2>(6.1359231515425647e-3f),
+                               bc<float2>(-3.1385246920140220f));
+        c[j] = make_float2(hw_cos(th.x), hw_cos(th.y));
+        s[j] = make_float2(hw_sin(th.x), hw_sin(th.y));
+    }
+}
+
+// Everything after the forward transform: Guo velocity, relaxation with the
+// source, noise, inverse transform delta f_i = w_i sum_k e_ki m_k / b_k, factored
+// into symmetric sums and differences.  m: the raw moments 3 .. 8 (general path
+// only).
+template <bool UNIT, typename V>
+__device__ __forceinline__ void collide_tail(V drho, V m1, V m2, const V m[6], V Fx, V Fy,
+                                             const KParams<scalar_t<V>> &p,
+                                             const uint32_t *__restrict__ rk, uint32_t site,
+                                             uint32_t step, V f[9]) {
+    using T = scalar_t<V>;
+    const V rho = vadd(bc<V>(p.rho0), drho);
+    const V inv_rho = inv_rho_of(rho);
+    const V jxh = vfma(bc<V>(T(0.5)), Fx, m1), jyh = vfma(bc<V>(T(0.5)), Fy, m2);   // rho u
+    const V ux = vmul(jxh, inv_rho), uy = vmul(jyh, inv_rho), nuy = vneg(uy);
+    // sums and differences of rho u u (q) and u F (p), each with one rounding of
+    // its x part
+    const V qs = vfma(jxh, ux, vmul(jyh, uy)), qd = vfma(jxh, ux, vmul(jyh, nuy));
+    const V ps = vfma(ux, Fx, vmul(uy, Fy)), pd = vfma(ux, Fx, vmul(nuy, Fy));
+    const V qxy = vmul(jxh, uy), pxy = vfma(ux, Fy, vmul(uy, Fx));
+    V m3, m4, m5, m6, m7, m8;
+    if (UNIT) {   // the general expressions with gamma = 0
+        m3 = vfma(bc<V>(T(3)), qs, vmul(bc<V>(T(3)), ps));
+        m4 = vadd(qd, pd);
+        m5 = vfma(bc<V>(T(0.5)), pxy, qxy);
+        m6 = m7 = m8 = bc<V>(T(0));
+    } else {
+        m3 = vfma(bc<V>(p.gamma_b), m[0], vfma(bc<V>(p.c3a), qs, vmul(bc<V>(p.c3b), ps)));
+        m4 = vfma(bc<V>(p.gamma), m[1], vfma(bc<V>(p.c4a), qd, vmul(bc<V>(p.c4b), pd)));
+        m5 = vfma(bc<V>(p.gamma), m[2], vfma(bc<V>(p.c5a), qxy, vmul(bc<V>(p.c5b), pxy)));
+        m6 = vmul(bc<V>(p.gamma_g), m[3]);
+        m7 = vmul(bc<V>(p.gamma_g), m[4]);
+        m8 = vmul(bc<V>(p.gamma_g), m[5]);
+    }
+    if (p.noise) {
+        V rad[3], c[3], s[3];
+        ring_noise(rho, p, rk, site, step, rad, c, s);
+        m3 = vfma(vmul(bc<V>(p.amp[0]), rad[0]), c[0], m3);
+        m4 = vfma(vmul(bc<V>(p.amp[1]), rad[0]), s[0], m4);
+        m5 = vfma(vmul(bc<V>(p.amp[2]), rad[1]), c[1], m5);
+        m6 = vfma(vmul(bc<V>(p.amp[3]), rad[1]), s[1], m6);
+        m7 = vfma(vmul(bc<V>(p.amp[4]), rad[2]), c[2], m7);
+        m8 = vfma(vmul(bc<V>(p.amp[5]), rad[2]), s[2], m8);
+    }
+    const V jx = vadd(m1, Fx), jy = vadd(m2, Fy);
+
+    f[0] = vfma(bc<V>(T(1.0 / 18.0)), m8,
+                vfma(bc<V>(T(-2.0 / 9.0)), m3, vmul(bc<V>(T(4.0 / 9.0)), drho)));
+    const V B = vfma(bc<V>(T(1.0 / 36.0)), vsub(m3, m8), vmul(bc<V>(T(1.0 / 9.0)), drho));
+    const V P = vfma(bc<V>(T(0.25)), m4, B), R = vfma(bc<V>(T(-0.25)), m4, B);
+    const V Q = vfma(bc<V>(T(-1.0 / 6.0)), m6, vmul(bc<V>(T(1.0 / 3.0)), jx));
+    const V Sq = vfma(bc<V>(T(-1.0 / 6.0)), m7, vmul(bc<V>(T(1.0 / 3.0)), jy));
+    f[1] = vadd(P, Q);
+    f[3] = vsub(P, Q);
+    f[2] = vadd(R, Sq);
+    f[4] = vsub(R, Sq);
+    const V D = vfma(bc<V>(T(1.0 / 72.0)), m8, vmul(bc<V>(T(1.0 / 36.0)), vadd(drho, m3)));
+    const V U = vfma(bc<V>(T(0.25)), m5, D), W = vfma(bc<V>(T(-0.25)), m5, D);
+    const V A = vadd(jx, m6), C = vadd(jy, m7);
+    const V X = vfma(bc<V>(T(1.0 / 12.0)), A, vmul(bc<V>(T(1.0 / 12.0)), C));
+    const V Y = vfma(bc<V>(T(1.0 / 12.0)), A, vmul(bc<V>(T(-1.0 / 12.0)), C));
+    f[5] = vadd(U, X);
+    f[7] = vsub(U, X);
+    f[6] = vsub(W, Y);
+    f[8] = vadd(W, Y);
+}
+
+// The unit-relaxation collision from the mass and momentum deviations alone.
+template <typename V>
+__device__ __forceinline__ void collide_unit_m(V drho, V m1, V m2, V Fx, V Fy,
+                                               const KParams<scalar_t<V>> &p,
+                                               const uint32_t *__restrict__ rk, uint32_t site,
+                                               uint32_t step, V f[9]) {
+    collide_tail<true, V>(drho, m1, m2, nullptr, Fx, Fy, p, rk, site, step, f);
 }
 
 // Collision of one site in the Hermite moment basis, Eq. (12):
@@ -75,144 +212,52 @@ __device__ __forceinline__ T sum9(const T g[9]) {
 // (1 - 1/2tau_k)(u F + F u) (BGK when every rate is 1/tau; bulk mode 3,
 // shear modes 4-5 and ghosts 6-8 may relax at their own rates), ghost modes
 // relaxed towards zero, momentum j + F
-// -> noise sqrt(mu rho b_k (1 - gamma^2)) z_k on modes 3..8 (one Philox
-// call, Box-Muller on a ring of 1024 angles) -> inverse
-// transform delta f_i = w_i sum_k e_ki m_k / b_k.  The inverse is factored
-// into symmetric sums and differences with the weights folded in.
-// UNIT: every relaxation rate is 1 (tau = tau_bulk = tau_ghost = 1, gamma = 0):
-// the non-conserved moments are replaced by their equilibrium, source and
-// noise, so m3..m8 of the pulled populations are not needed; the result is
-// bit-identical to the general path with gamma = 0.
-template <typename T>
-__device__ __forceinline__ void collide_tail(T drho, T m1, T m2, T m3, T m4, T m5, T m6, T m7,
-                                             T m8, T Fx, T Fy, const KParams<T> &p,
-                                             const uint32_t *__restrict__ rk, uint32_t site,
-                                             uint32_t step, T f[9], bool unit);
-
-// The step counter of the noise for a kernel launched with params p.
-template <typename T>
-__device__ __forceinline__ uint32_t step_of(const KParams<T> &p) {
-    return p.clock ? p.step + __ldg(p.clock) : p.step;
-}
-
-// Mass and momentum deviations of the pulled populations, with exactly the
-// arithmetic of the forward transform in collide (so that a kernel may keep
-// them instead of the nine populations on the unit-relaxation path).
-template <typename T>
-__device__ __forceinline__ void unit_moments(const T g[9], T &drho, T &m1, T &m2) {
-    const T e13 = g[1] - g[3], e24 = g[2] - g[4];
-    const T s13 = g[1] + g[3], s24 = g[2] + g[4];
-    const T d57 = g[5] - g[7], d86 = g[8] - g[6];
-    const T s57 = g[5] + g[7], s68 = g[6] + g[8];
-    const T sa = s13 + s24, sd = s57 + s68;
-    drho = g[0] + (sa + sd);
-    const T t1 = d57 + d86, t2 = d57 - d86;
-    m1 = e13 + t1;
-    m2 = e24 + t2;
-}
-
-// The unit-relaxation collision from the mass and momentum deviations alone.
-template <typename T>
-__device__ __forceinline__ void collide_unit_m(T drho, T m1, T m2, T Fx, T Fy, const KParams<T> &p,
-                                               const uint32_t *__restrict__ rk, uint32_t site,
-                                               uint32_t step, T f[9]) {
-    collide_tail<T>(drho, m1, m2, T(0), T(0), T(0), T(0), T(0), T(0), Fx, Fy, p, rk, site, step, f,
-                    true);
-}
-
-template <typename T, bool UNIT = false>
-__device__ __forceinline__ void collide(const T g[9], T Fx, T Fy, const KParams<T> &p,
+// -> noise sqrt(mu rho b_k (1 - gamma^2)) z_k on modes 3..8 -> inverse
+// transform.  FP32 kernels take collide_unit_m where p.unit (every relaxation
+// rate is 1: the non-conserved moments of the pulled populations are not
+// needed), this one elsewhere.
+template <typename V>
+__device__ __forceinline__ void collide(const V g[9], V Fx, V Fy, const KParams<scalar_t<V>> &p,
                                         const uint32_t *__restrict__ rk, uint32_t site,
-                                        uint32_t step, T f[9]) {
-    if constexpr (UNIT) {
-        T drho, m1, m2;
-        unit_moments(g, drho, m1, m2);
-        collide_unit_m(drho, m1, m2, Fx, Fy, p, rk, site, step, f);
-        return;
-    }
+                                        uint32_t step, V f[9]) {
+    using T = scalar_t<V>;
     // forward transform (integer coefficients, shared subexpressions)
-    const T e13 = g[1] - g[3], e24 = g[2] - g[4];
-    const T s13 = g[1] + g[3], s24 = g[2] + g[4];
-    const T d57 = g[5] - g[7], d86 = g[8] - g[6];
-    const T s57 = g[5] + g[7], s68 = g[6] + g[8];
-    const T sa = s13 + s24, sd = s57 + s68;
-    const T drho = g[0] + (sa + sd);
-    const T t1 = d57 + d86, t2 = d57 - d86;
-    const T m1 = e13 + t1;                                   // j_x
-    const T m2 = e24 + t2;                                   // j_y
-    const T m3 = fma(T(4), sd, fma(T(-2), g[0], sa));        // 3c^2 - 2
-    const T m4 = s13 - s24;                                  // cx^2 - cy^2
-    const T m5 = s57 - s68;                                  // cx cy
-    const T m6 = fma(T(2), t1, -e13);                        // (3c^2 - 4) cx
-    const T m7 = fma(T(2), t2, -e24);                        // (3c^2 - 4) cy
-    const T m8 = fma(T(8), sd, fma(T(-4), sa, g[0] + g[0])); // 9c^4 - 15c^2 + 2
-    collide_tail<T>(drho, m1, m2, m3, m4, m5, m6, m7, m8, Fx, Fy, p, rk, site, step, f, false);
+    const V e13 = vsub(g[1], g[3]), e24 = vsub(g[2], g[4]);
+    const V s13 = vadd(g[1], g[3]), s24 = vadd(g[2], g[4]);
+    const V d57 = vsub(g[5], g[7]), d86 = vsub(g[8], g[6]);
+    const V s57 = vadd(g[5], g[7]), s68 = vadd(g[6], g[8]);
+    const V sa = vadd(s13, s24), sd = vadd(s57, s68);
+    const V drho = vadd(g[0], vadd(sa, sd));
+    const V t1 = vadd(d57, d86), t2 = vsub(d57, d86);
+    const V m1 = vadd(e13, t1);                                              // j_x
+    const V m2 = vadd(e24, t2);                                              // j_y
+    V m[6];
+    m[0] = vfma(bc<V>(T(4)), sd, vfma(bc<V>(T(-2)), g[0], sa));              // 3c^2 - 2
+    m[1] = vsub(s13, s24);                                                   // cx^2 - cy^2
+    m[2] = vsub(s57, s68);                                                   // cx cy
+    m[3] = vfma(bc<V>(T(2)), t1, vneg(e13));                                 // (3c^2 - 4) cx
+    m[4] = vfma(bc<V>(T(2)), t2, vneg(e24));                                 // (3c^2 - 4) cy
+    m[5] = vfma(bc<V>(T(8)), sd, vfma(bc<V>(T(-4)), sa, vadd(g[0], g[0])));  // 9c^4 - 15c^2 + 2
+    collide_tail<false, V>(drho, m1, m2, m, Fx, Fy, p, rk, site, step, f);
 }
 
-// Everything after the forward transform: Guo velocity, relaxation with the
-// source, noise, inverse transform.  unit: every rate is 1 (m3 .. m8 unused).
-template <typename T>
-__device__ __forceinline__ void collide_tail(T drho, T m1, T m2, T m3, T m4, T m5, T m6, T m7,
-                                             T m8, T Fx, T Fy, const KParams<T> &p,
-                                             const uint32_t *__restrict__ rk, uint32_t site,
-                                             uint32_t step, T f[9], bool unit) {
-    const T rho = p.rho0 + drho;
-    const T inv_rho = inv_rho_of(rho);
-    const T jxh = fma(T(0.5), Fx, m1), jyh = fma(T(0.5), Fy, m2);   // rho u
-    const T ux = jxh * inv_rho, uy = jyh * inv_rho;
-    const T qxx = jxh * ux, qyy = jyh * uy, qxy = jxh * uy;          // rho u u
-    const T pxx = ux * Fx, pyy = uy * Fy, pxy = fma(ux, Fy, uy * Fx);
-    T m3s, m4s, m5s, m6s, m7s, m8s;
-    if (unit) {
-        m3s = fma(p.c3a, qxx + qyy, p.c3b * (pxx + pyy));
-        m4s = fma(p.c4a, qxx - qyy, p.c4b * (pxx - pyy));
-        m5s = fma(p.c5a, qxy, p.c5b * pxy);
-        m6s = m7s = m8s = T(0);
-    } else {
-        const T gs = p.gamma, gg = p.gamma_g;
-        m3s = fma(p.gamma_b, m3, fma(p.c3a, qxx + qyy, p.c3b * (pxx + pyy)));
-        m4s = fma(gs, m4, fma(p.c4a, qxx - qyy, p.c4b * (pxx - pyy)));
-        m5s = fma(gs, m5, fma(p.c5a, qxy, p.c5b * pxy));
-        m6s = gg * m6;
-        m7s = gg * m7;
-        m8s = gg * m8;
-    }
-    const T jxs = m1 + Fx, jys = m2 + Fy;
-
-    if (p.noise) {
-        // one Philox call per site and step: radius words r.x, r.y, r.z and
-        // three 10-bit angle indices of r.w (bits 0-9, 10-19, 20-29)
-        const uint4 r = philox4x32_10(make_uint4(site, step, p.replica, 0u), rk);
-        T c, sn, rad;
-        box_ring_polar(uniform01<T>(r.x), r.w & 1023u, rho, rad, c, sn);
-        m3s = fma(p.amp[0] * rad, c, m3s);
-        m4s = fma(p.amp[1] * rad, sn, m4s);
-        box_ring_polar(uniform01<T>(r.y), (r.w >> 10) & 1023u, rho, rad, c, sn);
-        m5s = fma(p.amp[2] * rad, c, m5s);
-        m6s = fma(p.amp[3] * rad, sn, m6s);
-        box_ring_polar(uniform01<T>(r.z), (r.w >> 20) & 1023u, rho, rad, c, sn);
-        m7s = fma(p.amp[4] * rad, c, m7s);
-        m8s = fma(p.amp[5] * rad, sn, m8s);
-    }
-
-    // inverse transform
-    f[0] = fma(T(1.0 / 18.0), m8s, fma(T(-2.0 / 9.0), m3s, T(4.0 / 9.0) * drho));
-    const T B = fma(T(1.0 / 36.0), m3s - m8s, T(1.0 / 9.0) * drho);
-    const T P = fma(T(0.25), m4s, B), R = fma(T(-0.25), m4s, B);
-    const T Q = fma(T(-1.0 / 6.0), m6s, T(1.0 / 3.0) * jxs);
-    const T Sq = fma(T(-1.0 / 6.0), m7s, T(1.0 / 3.0) * jys);
-    f[1] = P + Q;
-    f[3] = P - Q;
-    f[2] = R + Sq;
-    f[4] = R - Sq;
-    const T D = fma(T(1.0 / 72.0), m8s, T(1.0 / 36.0) * (drho + m3s));
-    const T U = fma(T(0.25), m5s, D), V = fma(T(-0.25), m5s, D);
-    const T A = T(1.0 / 12.0) * (jxs + m6s), Bd = T(1.0 / 12.0) * (jys + m7s);
-    const T X = A + Bd, Y = A - Bd;
-    f[5] = U + X;
-    f[7] = U - X;
-    f[6] = V - Y;
-    f[8] = V + Y;
+// Folded constants of KParams (any struct with its members) from the rates
+// 1 - 1/tau of the bulk, shear and ghost modes and the noise amplitudes:
+// m3: (1-gb) 3 rho u^2 + hb 6 u.F ; m4: (1-gs) rho (ux^2-uy^2) + hs 2 (uxFx-uyFy)
+// m5: (1-gs) rho ux uy + hs (ux Fy + uy Fx), h = (1 + gamma)/2 = 1 - 1/(2 tau).
+template <typename T, typename K>
+inline void fold_rates(K &k, double gb, double gs, double gg, const double amp[6]) {
+    k.unit = gb == 0.0 && gs == 0.0 && gg == 0.0;
+    k.gamma_b = (T)gb;
+    k.gamma = (T)gs;
+    k.gamma_g = (T)gg;
+    k.c3a = (T)(3.0 * (1.0 - gb));
+    k.c3b = (T)(3.0 * (1.0 + gb));
+    k.c4a = (T)(1.0 - gs);
+    k.c4b = (T)(1.0 + gs);
+    k.c5a = (T)(1.0 - gs);
+    k.c5b = (T)(0.5 * (1.0 + gs));
+    for (int i = 0; i < 6; ++i) k.amp[i] = (T)-amp[i];
 }
 
 template <typename T>
@@ -235,18 +280,7 @@ inline KParams<T> make_params(const StepArgs &a) {
     k.psi_c = (T)a.psi_c;
     k.psi_b = (T)a.psi_b;
     k.psi0 = (T)a.psi0;
-    k.gamma = (T)a.gamma;
-    k.gamma_b = (T)a.gamma_b;
-    k.gamma_g = (T)a.gamma_g;
-    // m3: (1-gb) 3 rho u^2 + hb 6 u.F ; m4: (1-gs) rho (ux^2-uy^2) + hs 2 (uxFx-uyFy)
-    // m5: (1-gs) rho ux uy + hs (ux Fy + uy Fx), h = (1 + gamma)/2 = 1 - 1/(2 tau)
-    k.c3a = (T)(3.0 * (1.0 - a.gamma_b));
-    k.c3b = (T)(3.0 * (1.0 + a.gamma_b));
-    k.c4a = (T)(1.0 - a.gamma);
-    k.c4b = (T)(1.0 + a.gamma);
-    k.c5a = (T)(1.0 - a.gamma);
-    k.c5b = (T)(0.5 * (1.0 + a.gamma));
-    for (int i = 0; i < 6; ++i) k.amp[i] = (T)a.noise_amp[i];
+    fold_rates<T>(k, a.gamma_b, a.gamma, a.gamma_g, a.noise_amp);
     for (int i = 0; i < 20; ++i) k.rk[i] = a.round_keys[i];
     return k;
 }

@@ -8,6 +8,7 @@
 #include <stdint.h>
 
 #include "lbsc_collide.cuh"
+#include "lbsc_strip.cuh"
 
 namespace lbsc {
 
@@ -21,12 +22,16 @@ struct EnsRep {
     int nx, ny, ldx, psi_kind;
     int noise;
     uint32_t replica;
-    float rho0, force_pref, psi_c, psi_b, psi0, gamma;
-    float c3a, c3b, c4a, c4b, c5a, c5b;
+    float rho0, force_pref, psi_c, psi_b, psi0;
+    float gamma_b, gamma, gamma_g, c3a, c3b, c4a, c4b, c5a, c5b;
     float amp[6];
+    int unit;
 };   // single relaxation time per replica (BGK)
+// One tile: the strip of columns from x0 of replica r, rows [y0, y1) in bands of h
+// rows (PairShape of the replica's width).
 struct EnsTile {
-    int r, x0, y0, y1;
+    int r, x0, y0, y1, h;
+    PairShape shape;
 };
 struct EnsClock {
     uint32_t t;
@@ -59,15 +64,16 @@ __device__ __forceinline__ void fill_tile_params(KParams<float> &sp, const EnsRe
     sp.psi_c = R.psi_c;
     sp.psi_b = R.psi_b;
     sp.psi0 = R.psi0;
+    sp.gamma_b = R.gamma_b;
     sp.gamma = R.gamma;
-    sp.gamma_b = R.gamma;
-    sp.gamma_g = R.gamma;
+    sp.gamma_g = R.gamma_g;
     sp.c3a = R.c3a;
     sp.c3b = R.c3b;
     sp.c4a = R.c4a;
     sp.c4b = R.c4b;
     sp.c5a = R.c5a;
     sp.c5b = R.c5b;
+    sp.unit = R.unit;
     for (int k = 0; k < 6; ++k) sp.amp[k] = R.amp[k];
 }
 

@@ -5,9 +5,9 @@
 // of Figs. 2-3 of arXiv:2212.07848) need many independent realisations; one
 // small lattice cannot fill a GB300 and a launch per replica per step is
 // launch-bound.  Here every step of every replica is one launch over a tile
-// list (replica, strip of 128 - 2H columns, row strip) sorted largest
-// replica first (the overlapped layout of the single-lattice kernel: 128
-// threads per CTA pull the strip and its halo columns);
+// list (replica, strip of columns, row strip) sorted largest replica first (the
+// strips of the single-lattice kernel, two columns per thread; a narrow replica's
+// tile holds several bands of rows);
 // each CTA copies its replica's parameters into shared memory and runs the
 // same per-strip code as the single-lattice kernel, so a replica evolves
 // bit-identically to a single lattice with the same seed and replica index.
@@ -39,15 +39,21 @@
 namespace lbsc {
 namespace {
 
-// OV: the overlapped layout (kStepTX threads, strips of kStepTX - 2H
-// columns); otherwise strips of kStepTX columns and a halo warp.
-template <int ORDER, bool OV>
-__global__ void __launch_bounds__(OV ? kStepTX : kStepTX + 32, OV ? (ORDER == 4 ? 8 : 5)
-                                                                  : (ORDER == 4 ? 6 : 4))
+// Threads per group (two columns each, step_pair) and groups per SM of a layout.
+__host__ __device__ constexpr int ens_threads(bool ov) { return ov ? 128 : 64; }
+__host__ __device__ constexpr int ens_minb(bool ov, int order) {
+    return (order == 4 ? 10 : 8) * 64 / ens_threads(ov);
+}
+
+// UM: 1 every replica takes the unit path (all rates 1), 0 none does, 2 each
+// replica by its own rates.  One strip variant per kernel (two for UM 2): more
+// inlined variants push the strip past the register budget that the launch bounds
+// leave, and it spills.
+template <int ORDER, bool OV, int UM, bool SAMPLE>
+__global__ void __launch_bounds__(ens_threads(OV), ens_minb(OV, ORDER))
 ens_step_kernel(const EnsRep *__restrict__ reps, const EnsTile *__restrict__ tiles, int ntiles,
-                EnsClock *clk, int *flag, const EnsKeys keys, int sk_every, long long sk_start) {
+                EnsClock *clk, int *flag, const EnsKeys keys) {
     __shared__ KParams<float> sp;
-    __shared__ int s_sample;
     __shared__ uint32_t s_t;
     __shared__ int s_cur;
     const EnsTile tile = tiles[blockIdx.x];
@@ -55,35 +61,24 @@ ens_step_kernel(const EnsRep *__restrict__ reps, const EnsTile *__restrict__ til
         const uint32_t t = __ldcg(&clk->t);
         const int cur = __ldcg(&clk->cur);
         const EnsRep &R = reps[tile.r];
-        const long long tn = (long long)t + 1;
-        const bool sample =
-            R.drho && sk_every > 0 && tn >= sk_start && (tn - sk_start) % sk_every == 0;
-        fill_tile_params(sp, R, tile, t, cur, sample, flag);
-        s_sample = sample ? 1 : 0;
+        fill_tile_params(sp, R, tile, t, cur, SAMPLE, flag);
         s_t = t;
         s_cur = cur;
     }
     __syncthreads();
     // replicas with every relaxation rate 1 (tau = 1) take the unit path,
     // which keeps only the conserved moments of the pulled rows
-    const bool unit = sp.gamma == 0.f;
-    if (OV) {
-        if (unit) {
-            if (s_sample) step_strip_ov<float, ORDER, true, false, true>(sp, keys.rk, tile.x0, tile.y0, tile.y1);
-            else step_strip_ov<float, ORDER, false, false, true>(sp, keys.rk, tile.x0, tile.y0, tile.y1);
-        } else {
-            if (s_sample) step_strip_ov<float, ORDER, true>(sp, keys.rk, tile.x0, tile.y0, tile.y1);
-            else step_strip_ov<float, ORDER, false>(sp, keys.rk, tile.x0, tile.y0, tile.y1);
-        }
+    constexpr int NT = ens_threads(OV);
+#define ENS_STRIP(U)                                                                           \
+    step_pair<ORDER, SAMPLE, false, U, NT>(sp, keys.rk, tile.shape, tile.x0, tile.y0, tile.h,  \
+                                           tile.y1)
+    if (UM == 2) {
+        if (sp.unit) ENS_STRIP(true);
+        else ENS_STRIP(false);
     } else {
-        if (unit) {
-            if (s_sample) step_strip<float, ORDER, true, false, true>(sp, keys.rk, tile.x0, tile.y0, tile.y1);
-            else step_strip<float, ORDER, false, false, true>(sp, keys.rk, tile.x0, tile.y0, tile.y1);
-        } else {
-            if (s_sample) step_strip<float, ORDER, true>(sp, keys.rk, tile.x0, tile.y0, tile.y1);
-            else step_strip<float, ORDER, false>(sp, keys.rk, tile.x0, tile.y0, tile.y1);
-        }
+        ENS_STRIP(UM == 1);
     }
+#undef ENS_STRIP
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
@@ -160,14 +155,10 @@ __device__ int wait_tiles(const uint32_t *tdone, const int *__restrict__ nbr, in
     }
 }
 
-// UM: 1 every replica takes the unit path (all rates 1), 0 none does, 2 each
-// replica by its own rates.  One strip variant per kernel (two for UM 2):
-// more inlined variants in the loop push the strip past the register budget
-// the launch bounds leave, and it spills.  The persistent launch never
-// samples; a sampling step runs through the per-step kernel.
+// UM as in ens_step_kernel.  The persistent launch never samples; a sampling step
+// runs through the per-step kernel.
 template <int ORDER, bool OV, int UM>
-__global__ void __launch_bounds__(OV ? kStepTX : kStepTX + 32, OV ? (ORDER == 4 ? 8 : 5)
-                                                                  : (ORDER == 4 ? 6 : 4))
+__global__ void __launch_bounds__(ens_threads(OV), ens_minb(OV, ORDER))
 ens_persist_kernel(const EnsRep *__restrict__ reps, const EnsTile *__restrict__ tiles,
                    int ntiles, const int *__restrict__ nbr_off, const int *__restrict__ nbr,
                    uint32_t *tdone, EnsCtl *ctl, EnsClock *clk, int *flag, const EnsKeys keys,
@@ -223,15 +214,15 @@ ens_persist_kernel(const EnsRep *__restrict__ reps, const EnsTile *__restrict__ 
         }
         __syncthreads();
         if (!s_go) break;
-#define ENS_STRIP(FN, U) FN<float, ORDER, false, true, U>(sp, keys.rk, s_tile.x0, s_tile.y0, s_tile.y1)
+        constexpr int NT = ens_threads(OV);
+#define ENS_STRIP(U)                                                                            \
+    step_pair<ORDER, false, true, U, NT>(sp, keys.rk, s_tile.shape, s_tile.x0, s_tile.y0,       \
+                                         s_tile.h, s_tile.y1)
         if (UM == 2) {
-            if (sp.gamma == 0.f) {
-                if (OV) ENS_STRIP(step_strip_ov, true); else ENS_STRIP(step_strip, true);
-            } else {
-                if (OV) ENS_STRIP(step_strip_ov, false); else ENS_STRIP(step_strip, false);
-            }
+            if (sp.unit) ENS_STRIP(true);
+            else ENS_STRIP(false);
         } else {
-            if (OV) ENS_STRIP(step_strip_ov, UM == 1); else ENS_STRIP(step_strip, UM == 1);
+            ENS_STRIP(UM == 1);
         }
 #undef ENS_STRIP
         if (threadIdx.x == 0) s_k[it ^ 1] = knext;
@@ -380,7 +371,7 @@ double psi_of(int kind, double p1, double p2, double rho) {
 void fill_rep_params(lb_ens *e, int r) {
     const lb_replica &q = e->reps[r];
     EnsRep &R = e->h_reps[r];
-    const double gam = 1.0 - 1.0 / q.tau, hs = 1.0 - 0.5 / q.tau;
+    const double gam = 1.0 - 1.0 / q.tau;
     R.psi_kind = e->psi_kind;
     R.noise = q.kT > 0.0 ? 1 : 0;
     R.replica = (uint32_t)r;
@@ -389,15 +380,10 @@ void fill_rep_params(lb_ens *e, int r) {
     R.psi0 = (float)psi_of(e->psi_kind, e->p1, e->p2, q.rho0);
     R.psi_c = e->psi_kind == LB_PSI_EXP ? (float)exp(-q.rho0) : R.psi0;
     R.psi_b = e->psi_kind == LB_PSI_EXP ? 0.0f : (float)e->p2;
-    R.gamma = (float)gam;
-    R.c3a = (float)(3.0 * (1.0 - gam));
-    R.c3b = (float)(6.0 * hs);
-    R.c4a = (float)(1.0 - gam);
-    R.c4b = (float)(2.0 * hs);
-    R.c5a = (float)(1.0 - gam);
-    R.c5b = (float)hs;
     const double mu = q.kT / kCs2;
-    for (int k = 0; k < 6; ++k) R.amp[k] = (float)sqrt(mu * kB[k] * (1.0 - gam * gam));
+    double amp[6];
+    for (int k = 0; k < 6; ++k) amp[k] = sqrt(mu * kB[k] * (1.0 - gam * gam));
+    fold_rates<float>(R, gam, gam, gam, amp);
 }
 
 void drop_graphs(lb_ens *e) {
@@ -510,9 +496,10 @@ int build_tiles(lb_ens *e) {
     for (int r : order) {
         if (e->is_res[r]) continue;   // advanced by the resident kernel
         const int nx = e->reps[r].nx, ny = e->reps[r].ny;
-        const int h = std::min(e->strip_h, ny);
-        const int cols = e->ov ? kStepTX - 2 * H : kStepTX;
-        const int nry = (ny + h - 1) / h, ncx = (nx + cols - 1) / cols;
+        const PairShape shape = pair_shape(nx, ens_threads(e->ov));
+        const int hb = std::min(e->strip_h, (ny + shape.bands - 1) / shape.bands);
+        const int h = hb * shape.bands, cols = shape.cols;
+        const int nry = (ny + h - 1) / h, ncx = shape.strips;
         const int base = (int)tiles.size();
         // strips whose cells the tiles of one row (column) strip read
         auto strips = [](int a0, int a1, int n, int w, int halo) {
@@ -530,7 +517,7 @@ int build_tiles(lb_ens *e) {
         for (int ry = 0; ry < nry; ++ry)
             for (int cx = 0; cx < ncx; ++cx) {
                 const int y0 = ry * h, x0 = cx * cols;
-                tiles.push_back({r, x0, y0, std::min(y0 + h, ny)});
+                tiles.push_back({r, x0, y0, std::min(y0 + h, ny), hb, shape});
                 for (int a : rset[ry])
                     for (int b : cset[cx]) nbr.push_back(base + a * ncx + b);
                 nbr_off.push_back((int)nbr.size());
@@ -569,7 +556,7 @@ cudaError_t launch_persist_t(lb_ens *e, int nsteps) {
                     &nsteps};
     const int grid = std::min(e->persist_grid, e->ntiles);
     return cudaLaunchCooperativeKernel((const void *)ens_persist_kernel<ORDER, OV, UM>,
-                                       dim3(grid), dim3(OV ? kStepTX : kStepTX + 32), args, 0,
+                                       dim3(grid), dim3(ens_threads(OV)), args, 0,
                                        e->stream);
 }
 
@@ -606,7 +593,7 @@ cudaError_t launch_persist_o(lb_ens *e, int nsteps) {
 cudaError_t persist_occupancy(lb_ens *e) {
     int per_sm = 0, nsm = 0;
     cudaError_t err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &per_sm, persist_fn(e), e->ov ? kStepTX : kStepTX + 32, 0);
+        &per_sm, persist_fn(e), ens_threads(e->ov), 0);
     if (err == cudaSuccess) err = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, e->dev);
     e->persist_grid = per_sm * nsm;
     return err;
@@ -631,27 +618,35 @@ cudaError_t launch_ens_persistent(lb_ens *e, int nsteps, bool sample_last) {
     return launch_ens_step(e, true);
 }
 
-// One step of every replica; `sample` also runs the S(k) sample of all
-// replicas (the step kernel then writes delta rho: the device decides from
-// its own step counter, which agrees with the host's).
-cudaError_t launch_ens_step(lb_ens *e, bool sample) {
-    const int sk_every = sample ? e->sk_every : 0;
-#define ENS_STEP(O, V, B)                                                                     \
-    ens_step_kernel<O, V><<<e->ntiles, B, 0, e->stream>>>(e->d_reps, e->d_tiles, e->ntiles,   \
-                                                          e->d_clk, e->d_flag, e->keys,       \
-                                                          sk_every, e->sk_start)
-    if (e->ntiles == 0) {
-        clock_advance_kernel<<<1, 1, 0, e->stream>>>(e->d_clk, 1);
-    } else if (e->ov) {
-        if (e->stencil == 4) ENS_STEP(4, true, kStepTX);
-        else if (e->stencil == 6) ENS_STEP(6, true, kStepTX);
-        else ENS_STEP(8, true, kStepTX);
+template <int ORDER, bool OV, int UM>
+void launch_ens_step_t(lb_ens *e, bool sample) {
+    if (sample)
+        ens_step_kernel<ORDER, OV, UM, true><<<e->ntiles, ens_threads(OV), 0, e->stream>>>(
+            e->d_reps, e->d_tiles, e->ntiles, e->d_clk, e->d_flag, e->keys);
+    else
+        ens_step_kernel<ORDER, OV, UM, false><<<e->ntiles, ens_threads(OV), 0, e->stream>>>(
+            e->d_reps, e->d_tiles, e->ntiles, e->d_clk, e->d_flag, e->keys);
+}
+template <int ORDER>
+void launch_ens_step_o(lb_ens *e, bool sample) {
+    if (e->ov) {
+        if (e->umode == 1) launch_ens_step_t<ORDER, true, 1>(e, sample);
+        else if (e->umode == 0) launch_ens_step_t<ORDER, true, 0>(e, sample);
+        else launch_ens_step_t<ORDER, true, 2>(e, sample);
     } else {
-        if (e->stencil == 4) ENS_STEP(4, false, kStepTX + 32);
-        else if (e->stencil == 6) ENS_STEP(6, false, kStepTX + 32);
-        else ENS_STEP(8, false, kStepTX + 32);
+        if (e->umode == 1) launch_ens_step_t<ORDER, false, 1>(e, sample);
+        else if (e->umode == 0) launch_ens_step_t<ORDER, false, 0>(e, sample);
+        else launch_ens_step_t<ORDER, false, 2>(e, sample);
     }
-#undef ENS_STEP
+}
+
+// One step of every replica; `sample` also runs the S(k) sample of all
+// replicas (the step kernel then writes delta rho).
+cudaError_t launch_ens_step(lb_ens *e, bool sample) {
+    if (e->ntiles == 0) clock_advance_kernel<<<1, 1, 0, e->stream>>>(e->d_clk, 1);
+    else if (e->stencil == 4) launch_ens_step_o<4>(e, sample);
+    else if (e->stencil == 6) launch_ens_step_o<6>(e, sample);
+    else launch_ens_step_o<8>(e, sample);
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess || !sample) return err;
     ens_rows_kernel<<<e->nrows, 512, (size_t)e->max_nx * sizeof(float2), e->stream>>>(e->d_reps,
@@ -815,10 +810,9 @@ int lb_ens_create(lb_ens **out, const lb_replica *reps, int nrep, int psi_kind, 
         err = cudaMemcpy(e->d_ctl, &c0, sizeof(EnsCtl), cudaMemcpyHostToDevice);
     }
     {
-        // a replica takes the unit path when its rate gamma rounds to 0 in
-        // FP32, the test the kernels make
+        // a replica takes the unit path when its rates are 1 (fold_rates)
         int nunit = 0;
-        for (int r = 0; r < nrep; ++r) nunit += (float)(1.0 - 1.0 / reps[r].tau) == 0.0f;
+        for (int r = 0; r < nrep; ++r) nunit += 1.0 - 1.0 / reps[r].tau == 0.0;
         e->umode = nunit == nrep ? 1 : nunit == 0 ? 0 : 2;
     }
     if (err == cudaSuccess) err = persist_occupancy(e);
@@ -975,9 +969,10 @@ int lb_ens_set_kernel(lb_ens *e, int mode) {
     ENS_CHECK(cudaSetDevice(e->dev));
     ENS_CHECK(cudaStreamSynchronize(e->stream));
     e->kernel_mode = mode;
-    // AUTO: the halo-warp layout.  Replica widths are powers of two up to a
-    // few hundred columns, where the overlapped layout's last strip holds
-    // only a few columns (256 replicas of {64..512}^2: 61 against 56 GLUPS).
+    // AUTO: 64-thread tiles.  Replica widths are powers of two up to a few hundred
+    // columns, where the wider tile measured within 3% (256 replicas of
+    // {64..512}^2, persistent: 256 against 250 us a step, both 336 us with one column
+    // per thread) but is slower for 32^2.
     e->ov = mode == LB_KERNEL_OVERLAP;
     ENS_CHECK(persist_occupancy(e));
     return build_tiles(e);

@@ -7,9 +7,9 @@
 
 namespace lbsc {
 
-// Launch shape of the fused step: one thread per lattice column inside a
-// strip of kStepTX columns; each CTA sweeps strip_h rows of its strip.
-constexpr int kStepTX = 128;
+// How a step kernel cuts the lattice (StepArgs::layout): strips swept by groups of
+// 64 or 128 threads, or tiles (FP64 lattices always run in tiles).
+constexpr int kLayoutNarrow = 0, kLayoutWide = 1, kLayoutTile = 2;
 
 // Bits of the device status flag read by lb_sync.
 constexpr int LB_STEP_NONFINITE = 1;
@@ -32,7 +32,7 @@ struct StepArgs {
     void *drho_out;       // delta rho [ny][nx] of the new state, or nullptr
     int *flag;            // LB_STEP_* bits (non-finite value, wait timeout)
     int nx, ny;
-    int strip_h;          // rows swept by one CTA
+    int strip_h;          // rows of a strip (of a band of it: PairShape)
     double rho0;          // reference density of the stored deviations
     double force_pref;    // -G c_s^2
     double psi_kind;      // 0, 1, 2 (kept as double for packing)
@@ -48,7 +48,7 @@ struct StepArgs {
     uint32_t replica;     // counter word 2
     int noise;            // kT > 0
     long long wait_ns;    // staged kernel: bound on an mbarrier wait (< 0: default)
-    int layout;           // plain kernel: 0 = halo warp, 1 = overlapped strips
+    int layout;           // kLayout*
     const uint32_t *clock;  // device step counter: the noise counter is *clock + step (or null)
 };
 
@@ -63,6 +63,8 @@ struct SkArgs {
 };
 
 cudaError_t launch_step(int precision, int stencil, const StepArgs &a, cudaStream_t s);
+bool tile_is_faster(int nx, int ny, bool unit);
+int strip_rows(int nx, int ny, int layout, bool unit);
 bool tma_eligible(int precision, int nx, int ny);
 bool tma_encode_maps(TmaMaps *m, void *buf0, void *buf1, int nx, int ny);
 // src_buf: index (0/1) of the buffer holding the current state.

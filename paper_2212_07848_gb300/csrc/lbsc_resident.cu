@@ -90,8 +90,7 @@ template <int ORDER, bool UNIT>
 __device__ __forceinline__ void res_sweep(const KParams<float> &p, const uint32_t *__restrict__ rk,
                                           float *sm, float *ring, uint32_t P, int nx, int rows,
                                           int band, int hb, int tx, int ybase) {
-    using S = Stencil<ORDER>;
-    constexpr int H = S::H;
+    constexpr int H = Stencil<ORDER>::H;
     constexpr int RING = res_ring<ORDER>();
     const int y0 = band * hb, y1 = y0 + hb;
     const int xm = (tx - 1) & (nx - 1), xp = (tx + 1) & (nx - 1);
@@ -123,7 +122,7 @@ __device__ __forceinline__ void res_sweep(const KParams<float> &p, const uint32_
             pull_sm(sm, P, nx, tx, xm, xp, row_of(yc - 1), row_of(yc), row_of(yc + 1), gn);
         }
         const float s9 = sum9(g);
-        ring[slot * nx + tx] = delta_psi<float>(s9, p.psi_kind, rho0, p.psi_c, p.psi_b);
+        ring[slot * nx + tx] = delta_psi(s9, p.psi_kind, rho0, p.psi_c, p.psi_b);
 #pragma unroll
         for (int r = 0; r < H; ++r)
 #pragma unroll
@@ -139,25 +138,21 @@ __device__ __forceinline__ void res_sweep(const KParams<float> &p, const uint32_
         if (it < 2 * H) continue;
 
         const int yr = y0 - 2 * H + it;   // the row collided, local
-        float sx = 0.f, sy = 0.f;
-#pragma unroll
-        for (int a = 0; a < S::N; ++a) {
-            const HalfVec hv = S::v(a);
-            const float dpl = ring[((it - H + hv.ey) & (RING - 1)) * nx + ((tx + hv.ex) & (nx - 1))];
-            const float dmi = ring[((it - H - hv.ey) & (RING - 1)) * nx + ((tx - hv.ex) & (nx - 1))];
-            const float d = float(hv.w) * (dpl - dmi);
-            if (hv.ex != 0) sx += float(hv.ex) * d;
-            if (hv.ey != 0) sy += float(hv.ey) * d;
-        }
-        const float psic = p.psi0 + ring[((it - H) & (RING - 1)) * nx + tx];
-        const float Fx = p.force_pref * psic * sx;
-        const float Fy = p.force_pref * psic * sy;
+        float sx, sy;
+        force_sums<ORDER>(
+            [&](int ex, int ey) {
+                return ring[((it - H + ey) & (RING - 1)) * nx + ((tx + ex) & (nx - 1))];
+            },
+            sx, sy);
+        const float psic = vadd(p.psi0, ring[((it - H) & (RING - 1)) * nx + tx]);
+        const float pf = vmul(p.force_pref, psic);
+        const float Fx = vmul(pf, sx), Fy = vmul(pf, sy);
 
         float f[9];
         const int yg = ybase + yr;
         const uint32_t site = (uint32_t)tx + (uint32_t)nx * (uint32_t)yg;
         if constexpr (UNIT) collide_unit_m(q[0][1], q[0][2], q[0][3], Fx, Fy, p, rk, site, p.step, f);
-        else collide<float, false>(q[0], Fx, Fy, p, rk, site, p.step, f);
+        else collide<float>(q[0], Fx, Fy, p, rk, site, p.step, f);
         float *w = sm + yr * nx + tx;
 #pragma unroll
         for (int i = 0; i < 9; ++i) w[i * P] = f[i];
@@ -192,13 +187,13 @@ ens_resident_kernel(const EnsRep *__restrict__ reps, const int *__restrict__ lis
     if (threadIdx.x == 0) {
         s_t0 = __ldcg(&clk->t);
         s_cur = __ldcg(&clk->cur);
-        const EnsTile whole = {0, 0, 0, hb};
+        const EnsTile whole = {0, 0, 0, hb, hb, {}};
         fill_tile_params(sp, R, whole, s_t0, s_cur, false, flag);
     }
     __syncthreads();
     const uint32_t t0 = s_t0;
     const int cur = s_cur;
-    const bool unit = sp.gamma == 0.f;   // every rate 1: the unit path
+    const bool unit = sp.unit != 0;   // every rate 1: the unit path
     const uint32_t gplane = (uint32_t)nx * ny;
     const uint32_t n4 = (uint32_t)rows * nx / 4;   // float4 of a plane's own rows
     {

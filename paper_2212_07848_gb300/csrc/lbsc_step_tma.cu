@@ -30,7 +30,7 @@ namespace lbsc {
 
 namespace {
 
-constexpr int kTX = kStepTX;            // interior columns per CTA (128)
+constexpr int kTX = 128;                // interior columns per CTA
 constexpr int kBox = kTX + 8;           // columns per staged row: x0-4 .. x0+131
 constexpr int kSlot = 1248;             // floats per ring slot: 9 x 136 = 1224 padded to 128 B
 constexpr uint64_t kWaitNs = 2000000000ull;   // default bound on a wait: 2 s
@@ -141,8 +141,7 @@ __global__ void __launch_bounds__(kTX + 32)
 step_kernel_tma(const __grid_constant__ CUtensorMap tm_src,
                 const __grid_constant__ CUtensorMap tm_dst, const KParams<float> p,
                 const unsigned long long wait_ns) {
-    using S = Stencil<ORDER>;
-    constexpr int H = S::H;
+    constexpr int H = Stencil<ORDER>::H;
     using Cfg = TmaCfg<H>;
     constexpr int R = Cfg::R;
     constexpr int PR = Cfg::PSI_RING;
@@ -246,7 +245,7 @@ step_kernel_tma(const __grid_constant__ CUtensorMap tm_src,
         if (interior || halo) {
             float g[9];
             pull_smem(slot_of(it) + col, slot_of(it + 1) + col, slot_of(it + 2) + col, g);
-            spsi[pslot * W + pcol] = delta_psi<float>(sum9(g), p.psi_kind, rho0, p.psi_c, p.psi_b);
+            spsi[pslot * W + pcol] = delta_psi(sum9(g), p.psi_kind, rho0, p.psi_c, p.psi_b);
         }
         // the store of the row collided in the previous iteration must have
         // read its staging buffer before that buffer is written again
@@ -270,23 +269,24 @@ step_kernel_tma(const __grid_constant__ CUtensorMap tm_src,
 
         // ---- collide row yr ------------------------------------------------
         const int yr = y0 + it - 2 * H;
-        float sx = 0.f, sy = 0.f;
-#pragma unroll
-        for (int a = 0; a < S::N; ++a) {
-            const HalfVec hv = S::v(a);
-            const float dpl = spsi[((it - H + hv.ey) & (PR - 1)) * W + pcol + hv.ex];
-            const float dmi = spsi[((it - H - hv.ey) & (PR - 1)) * W + pcol - hv.ex];
-            const float d = float(hv.w) * (dpl - dmi);
-            if (hv.ex != 0) sx += float(hv.ex) * d;
-            if (hv.ey != 0) sy += float(hv.ey) * d;
-        }
-        const float psic = p.psi0 + spsi[((it - H) & (PR - 1)) * W + pcol];
-        const float Fx = p.force_pref * psic * sx;
-        const float Fy = p.force_pref * psic * sy;
+        float sx, sy;
+        force_sums<ORDER>(
+            [&](int ex, int ey) { return spsi[((it - H + ey) & (PR - 1)) * W + pcol + ex]; }, sx,
+            sy);
+        const float psic = vadd(p.psi0, spsi[((it - H) & (PR - 1)) * W + pcol]);
+        const float pf = vmul(p.force_pref, psic);
+        const float Fx = vmul(pf, sx), Fy = vmul(pf, sy);
 
         float g[9], f[9];
         pull_smem(slot_of(it - H) + col, slot_of(it - H + 1) + col, slot_of(it - H + 2) + col, g);
-        collide(g, Fx, Fy, p, p.rk, (uint32_t)(x0 + tx) + (uint32_t)nx * (uint32_t)yr, step_of(p), f);
+        const uint32_t site = (uint32_t)(x0 + tx) + (uint32_t)nx * (uint32_t)yr;
+        if (p.unit) {
+            float drho, m1, m2;
+            unit_moments(g, drho, m1, m2);
+            collide_unit_m(drho, m1, m2, Fx, Fy, p, p.rk, site, step_of(p), f);
+        } else {
+            collide<float>(g, Fx, Fy, p, p.rk, site, step_of(p), f);
+        }
         float *st = stage + (it & 1) * 9 * kTX + tx;
 #pragma unroll
         for (int i = 0; i < 9; ++i) st[i * kTX] = f[i];
