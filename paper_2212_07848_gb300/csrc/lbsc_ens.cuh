@@ -87,7 +87,7 @@ struct ResLaunch {
     int nres;
     int nx, ny;             // the shape (nx in {32, 64, 128})
     int C;                  // CTAs per replica (cluster size: 1, 2, 4 or 8)
-    int hb;                 // rows per band (one thread per column and band)
+    bool unit;              // every replica of the list takes the unit path
     int stencil;            // 4, 6, 8
     EnsClock *clk;
     int *flag;
@@ -95,13 +95,13 @@ struct ResLaunch {
     int nsteps;
     int sample;             // the window's last step writes delta rho
 };
-// Dynamic shared memory of one CTA holding `rows` rows of nx columns in
-// bands of hb rows, or 0 if the shape is not supported.
-size_t resident_smem(int nx, int rows, int hb, int stencil);
-// Opt the kernel of (stencil, C) in to `smem` bytes of dynamic shared memory.
+// Dynamic shared memory of one CTA holding `rows` rows of nx columns, or 0 if the
+// shape is not supported.
+size_t resident_smem(int nx, int rows, int stencil);
+// Opt the kernels of (stencil, C) in to `smem` bytes of dynamic shared memory.
 cudaError_t resident_prepare(int stencil, int C, size_t smem);
 // Clusters of C CTAs (CTAs per SM when C = 1) that can be resident at once.
-int resident_max_clusters(int stencil, int C, int nx, int rows, int hb, size_t smem);
+int resident_max_clusters(int stencil, int C, int nx, int rows, bool unit, size_t smem);
 cudaError_t launch_ens_resident(const ResLaunch &a, cudaStream_t s);
 
 }  // namespace lbsc

@@ -295,9 +295,10 @@ size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 
 using namespace lbsc;
 
-// Resident replicas of one shape: C CTAs of hb-row bands per replica.
+// Resident replicas of one shape and path: C CTAs per replica.
 struct ResClass {
-    int nx, ny, C, hb;
+    int nx, ny, C;
+    bool unit;
     size_t smem;
     std::vector<int> reps;
     int *d_list = nullptr;
@@ -392,12 +393,10 @@ void drop_graphs(lb_ens *e) {
     e->graph_plain = e->graph_window = nullptr;
 }
 
-// Tiles of 128 columns x strip rows, largest replicas first.
 // Launch shape of a resident replica of nx x ny sites: the fewest CTAs per
-// replica (C, at most max_c) and then the shortest bands (hb) whose shared
-// memory fits one CTA and whose clusters can be resident; false if there is
-// none.
-bool resident_shape(const lb_ens *e, int nx, int ny, int max_c, ResClass *out) {
+// replica (C, at most max_c) whose shared memory fits one CTA and whose clusters
+// can be resident; false if there is none.
+bool resident_shape(const lb_ens *e, int nx, int ny, bool unit, int max_c, ResClass *out) {
     int optin = 0;
     if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, e->dev) !=
         cudaSuccess)
@@ -406,35 +405,31 @@ bool resident_shape(const lb_ens *e, int nx, int ny, int max_c, ResClass *out) {
     for (int c : {1, 2, 4, 8}) {
         if (c > max_c || ny % c) continue;
         const int rows = ny / c;
-        for (int hb : {8, 16, 32}) {
-            if (rows % hb) continue;
-            const size_t sm = resident_smem(nx, rows, hb, e->stencil);
-            if (!sm || sm > limit) continue;
-            if (resident_prepare(e->stencil, c, limit) != cudaSuccess) {
-                cudaGetLastError();
-                return false;
-            }
-            if (resident_max_clusters(e->stencil, c, nx, rows, hb, sm) < 1) {
-                cudaGetLastError();
-                continue;
-            }
-            out->nx = nx;
-            out->ny = ny;
-            out->C = c;
-            out->hb = hb;
-            out->smem = sm;
-            return true;
+        const size_t sm = resident_smem(nx, rows, e->stencil);
+        if (!sm || sm > limit) continue;
+        if (resident_prepare(e->stencil, c, limit) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
         }
+        if (resident_max_clusters(e->stencil, c, nx, rows, unit, sm) < 1) {
+            cudaGetLastError();
+            continue;
+        }
+        out->nx = nx;
+        out->ny = ny;
+        out->C = c;
+        out->unit = unit;
+        out->smem = sm;
+        return true;
     }
     return false;
 }
 
 // Which replicas live in shared memory (resident_mode): none; every one
 // whose shape allows it; or, AUTO, all of them when each fits one CTA.
-// AUTO leaves out the clusters (128^2 over four CTAs measured 42 against 63
-// GLUPS tiled: a tile already fills its 128 columns, clusters of four
-// 200 KB CTAs leave SMs of each GPC idle and each step waits at two cluster
-// barriers) and mixed ensembles (the resident launch runs before the tiles,
+// AUTO leaves out the clusters (128^2 over four CTAs measured 64 against 83
+// GLUPS tiled: clusters of four 180 KB CTAs leave SMs of each GPC idle and each
+// step waits at two cluster barriers) and mixed ensembles (the resident launch runs before the tiles,
 // so its few CTAs would hold up the rest of the GPU).
 int setup_resident(lb_ens *e) {
     for (auto &c : e->rclasses) cudaFree(c.d_list);
@@ -447,14 +442,15 @@ int setup_resident(lb_ens *e) {
     int n = 0;
     for (int r = 0; r < e->nrep; ++r) {
         const int nx = e->reps[r].nx, ny = e->reps[r].ny;
-        const long key = (long)nx * 1000003L + ny;
+        const bool unit = e->h_reps[r].unit != 0;
+        const long key = ((long)nx * 1000003L + ny) * 2 + (unit ? 1 : 0);
         int k = -2;
         for (const auto &t : tried)
             if (t.first == key) k = t.second;
         if (k == -2) {
             ResClass c;
             const int max_c = e->resident_mode == LB_ENS_RESIDENT_AUTO ? 1 : 8;
-            if (resident_shape(e, nx, ny, max_c, &c)) {
+            if (resident_shape(e, nx, ny, unit, max_c, &c)) {
                 cls.push_back(c);
                 k = (int)cls.size() - 1;
             } else {
@@ -676,7 +672,7 @@ cudaError_t launch_window(lb_ens *e, int steps, bool sample_last) {
         a.nx = c.nx;
         a.ny = c.ny;
         a.C = c.C;
-        a.hb = c.hb;
+        a.unit = c.unit;
         a.stencil = e->stencil;
         a.clk = e->d_clk;
         a.flag = e->d_flag;

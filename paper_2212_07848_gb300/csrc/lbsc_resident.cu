@@ -8,26 +8,27 @@
 // at a sampling step: a window of n steps moves 72 B per site once instead
 // of n times.
 //
-// Layout of one CTA (rows [rank R, rank R + R) of its replica, R = ny / C):
-// the nine population planes [9][Rtot][nx], Rtot = R + (nb + 1)(H + 1) --
-// the R own rows, then nb + 1 blocks of H + 1 copied rows -- and nb rings of
-// delta psi rows.  The CTA is nb bands of hb rows, one thread per column and
-// band.  Each band sweeps its rows like a strip of the global kernel (pull
-// one row ahead, delta psi into its ring, collide H rows behind) and writes
-// the new populations in place.  All bands advance in lock step, one barrier
-// per row, and in-place writes are safe because
-//  * a band reads each of its own rows at least H rows before it writes it;
-//  * a band pulls its lower halo (the last H + 1 rows of the band below)
-//    at the start of its sweep, before that band writes them at the end;
-//  * the first H + 1 rows of the band above are written at the start of the
-//    sweep but pulled at the end, so they are copied before the sweep, each
-//    step; so are the H + 1 rows below the CTA's lowest band, which belong
-//    to the previous CTA of the cluster (to the CTA itself when C = 1).
-// Copies from another CTA are distributed-shared-memory loads between two
-// cluster barriers: one after the previous step's writes, one before this
-// step's.  The arithmetic, summation order and Philox counters are those of
-// the tile path, so a resident replica evolves bit-identically to a single
-// lattice with the same seed and replica index.
+// Layout of one CTA (rows [rank R, rank R + R) of its replica, R = ny / C): the nine
+// population planes [9][R][nx] and the pseudopotential deviations of its rows with
+// H halo rows and two halo columns on each side, kept twice (see step_pair).  A
+// step is two phases with a barrier after each.  First every thread pulls its
+// pairs of neighbouring sites, writes their delta psi (and the copies of it that
+// the halo of its own or a neighbouring CTA needs) and keeps of the populations what
+// the collision reads: mass and momentum on the unit-relaxation path, all nine
+// otherwise.  Every read of the old state is then done, so the second phase
+// collides and writes the new populations in place.  No site is computed twice and
+// nothing is copied.  With C > 1 the rows beyond the CTA's are read, and the halo rows
+// written, through distributed shared memory, and the barriers are the cluster's.
+// The arithmetic, summation order and Philox counters are those of the tile path,
+// so a resident replica evolves bit-identically to a single lattice with the same
+// seed and replica index.
+//
+// Bound by issue and resident warps: 64^2 on the unit path runs 32 warps an SM at 64
+// registers.  1024 x 64^2: 81 GLUPS (56 with bands of rows swept in lock step, one
+// column per thread at 16 warps an SM, which pulled ten rows for eight and copied
+// the boundary rows every step); 4096 x 32^2: 93 (60).
+// 512 and 768 threads of more registers measured 74; the general path is faster at
+// 512 (63) than at 384 (51).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -37,7 +38,10 @@
 namespace lbsc {
 namespace {
 
-constexpr int kResMaxThreads = 512;
+// Most sites per CTA, threads per CTA and pairs per thread of a path: the unit path
+// holds three values of a pair across the barrier, the general path eighteen.
+constexpr int kResMaxSites = 4096;
+__host__ __device__ constexpr int res_threads(bool unit) { return unit ? 1024 : 512; }
 
 __device__ __forceinline__ uint32_t cluster_rank() {
     uint32_t r;
@@ -50,13 +54,20 @@ __device__ __forceinline__ void cluster_sync() {
         "barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 // The float at the offset of `p` in the shared memory of cluster CTA `rank`.
-__device__ __forceinline__ float ld_cluster(const float *p, uint32_t rank) {
+__device__ __forceinline__ uint32_t map_cluster(const float *p, uint32_t rank) {
     const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
     uint32_t ra;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(rank));
+    return ra;
+}
+__device__ __forceinline__ float ld_cluster(const float *p, uint32_t rank) {
     float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(ra) : "memory");
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(map_cluster(p, rank))
+                 : "memory");
     return v;
+}
+__device__ __forceinline__ void st_cluster(float *p, uint32_t rank, float v) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(map_cluster(p, rank)), "f"(v) : "memory");
 }
 template <int C>
 __device__ __forceinline__ void sync_all() {
@@ -64,114 +75,16 @@ __device__ __forceinline__ void sync_all() {
     else __syncthreads();
 }
 
-template <int ORDER>
-__host__ __device__ constexpr int res_ring() {
-    return Stencil<ORDER>::H == 1 ? 4 : 8;   // >= 2H + 2 rows, power of two
-}
-
-// Pull of one site from shared memory, the streaming of the global pull:
-// rows rm, rc, rp hold y - 1, y, y + 1 (shared-memory row indices).
-__device__ __forceinline__ void pull_sm(const float *sm, uint32_t P, int nx, int xc, int xm,
-                                        int xp, int rm, int rc, int rp, float g[9]) {
-    const float *c = sm + rc * nx, *m = sm + rm * nx, *q = sm + rp * nx;
-    g[0] = c[xc];
-    g[1] = c[P + xm];
-    g[2] = m[2u * P + xc];
-    g[3] = c[3u * P + xp];
-    g[4] = q[4u * P + xc];
-    g[5] = m[5u * P + xm];
-    g[6] = m[6u * P + xp];
-    g[7] = q[7u * P + xp];
-    g[8] = q[8u * P + xm];
-}
-
-// One step of one band: rows [y0, y0 + hb) of the CTA, in place.
-template <int ORDER, bool UNIT>
-__device__ __forceinline__ void res_sweep(const KParams<float> &p, const uint32_t *__restrict__ rk,
-                                          float *sm, float *ring, uint32_t P, int nx, int rows,
-                                          int band, int hb, int tx, int ybase) {
-    constexpr int H = Stencil<ORDER>::H;
-    constexpr int RING = res_ring<ORDER>();
-    const int y0 = band * hb, y1 = y0 + hb;
-    const int xm = (tx - 1) & (nx - 1), xp = (tx + 1) & (nx - 1);
-    // shared-memory row of local row ys as this band pulls it
-    auto row_of = [&](int ys) {
-        if (ys >= y1) return rows + (H + 1) * (1 + band) + (ys - y1);
-        if (ys < 0) return rows + (ys + H + 1);
-        return ys;
-    };
-    const float rho0 = p.rho0;
-    constexpr int NQ = UNIT ? 4 : 9;
-    float q[H + 1][NQ];
-#pragma unroll
-    for (int r = 0; r <= H; ++r)
-#pragma unroll
-        for (int i = 0; i < NQ; ++i) q[r][i] = 0.f;
-
-    const int it_end = hb + 2 * H;
-    float gn[9];
-    pull_sm(sm, P, nx, tx, xm, xp, row_of(y0 - H - 1), row_of(y0 - H), row_of(y0 - H + 1), gn);
-#pragma unroll 2
-    for (int it = 0; it < it_end; ++it) {
-        const int slot = it & (RING - 1);
-        float g[9];
-#pragma unroll
-        for (int i = 0; i < 9; ++i) g[i] = gn[i];
-        if (it + 1 < it_end) {
-            const int yc = y0 - H + it + 1;
-            pull_sm(sm, P, nx, tx, xm, xp, row_of(yc - 1), row_of(yc), row_of(yc + 1), gn);
-        }
-        const float s9 = sum9(g);
-        ring[slot * nx + tx] = delta_psi(s9, p.psi_kind, rho0, p.psi_c, p.psi_b);
-#pragma unroll
-        for (int r = 0; r < H; ++r)
-#pragma unroll
-            for (int i = 0; i < NQ; ++i) q[r][i] = q[r + 1][i];
-        if constexpr (UNIT) {
-            q[H][0] = s9;
-            unit_moments(g, q[H][1], q[H][2], q[H][3]);
-        } else {
-#pragma unroll
-            for (int i = 0; i < 9; ++i) q[H][i] = g[i];
-        }
-        __syncthreads();
-        if (it < 2 * H) continue;
-
-        const int yr = y0 - 2 * H + it;   // the row collided, local
-        float sx, sy;
-        force_sums<ORDER>(
-            [&](int ex, int ey) {
-                return ring[((it - H + ey) & (RING - 1)) * nx + ((tx + ex) & (nx - 1))];
-            },
-            sx, sy);
-        const float psic = vadd(p.psi0, ring[((it - H) & (RING - 1)) * nx + tx]);
-        const float pf = vmul(p.force_pref, psic);
-        const float Fx = vmul(pf, sx), Fy = vmul(pf, sy);
-
-        float f[9];
-        const int yg = ybase + yr;
-        const uint32_t site = (uint32_t)tx + (uint32_t)nx * (uint32_t)yg;
-        if constexpr (UNIT) collide_unit_m(q[0][1], q[0][2], q[0][3], Fx, Fy, p, rk, site, p.step, f);
-        else collide<float>(q[0], Fx, Fy, p, rk, site, p.step, f);
-        float *w = sm + yr * nx + tx;
-#pragma unroll
-        for (int i = 0; i < 9; ++i) w[i * P] = f[i];
-        if (p.drho_out) {
-            if constexpr (UNIT) p.drho_out[site] = q[0][0];
-            else p.drho_out[site] = sum9(q[0]);
-        }
-        if (!isfinite(f[1] + f[5])) atomicOr(p.flag, LB_STEP_NONFINITE);
-    }
-}
-
-// `nsteps` steps of every replica in `list` (one shape), C CTAs per replica.
-template <int ORDER, int C>
-__global__ void __launch_bounds__(kResMaxThreads)
+// `nsteps` steps of every replica in `list` (one shape, all of them on the unit
+// path or none), C CTAs per replica.
+template <int ORDER, int C, bool UNIT>
+__global__ void __launch_bounds__(res_threads(UNIT))
 ens_resident_kernel(const EnsRep *__restrict__ reps, const int *__restrict__ list,
                     const EnsClock *__restrict__ clk, int *flag, const EnsKeys keys, int nsteps,
-                    int sample, int hb) {
+                    int sample) {
     constexpr int H = Stencil<ORDER>::H;
-    constexpr int RING = res_ring<ORDER>();
+    constexpr int NP = (kResMaxSites / 2 + res_threads(UNIT) - 1) / res_threads(UNIT);   // pairs a thread
+    constexpr int NQ = UNIT ? 3 : 9;
     extern __shared__ __align__(16) float sm[];
     __shared__ KParams<float> sp;
     __shared__ uint32_t s_t0;
@@ -179,23 +92,20 @@ ens_resident_kernel(const EnsRep *__restrict__ reps, const int *__restrict__ lis
     const uint32_t rank = C > 1 ? cluster_rank() : 0u;
     const EnsRep &R = reps[list[blockIdx.x / C]];
     const int nx = R.nx, ny = R.ny;
-    const int rows = ny / C, nb = rows / hb;
-    const uint32_t P = (uint32_t)(rows + (nb + 1) * (H + 1)) * nx;   // plane stride
-    const int tx = threadIdx.x & (nx - 1), band = threadIdx.x / nx;
-    const int ybase = (int)rank * rows;
-    float *ring = sm + 9 * P + band * RING * nx;
+    const int rows = ny / C, ybase = (int)rank * rows;
+    const uint32_t P = (uint32_t)rows * nx;                    // plane stride
+    const int W = nx + 4;
+    float *sa = sm + 9 * P, *sb = sa + (rows + 2 * H) * W;     // rows -H .. rows + H - 1
     if (threadIdx.x == 0) {
         s_t0 = __ldcg(&clk->t);
         s_cur = __ldcg(&clk->cur);
-        const EnsTile whole = {0, 0, 0, hb, hb, {}};
-        fill_tile_params(sp, R, whole, s_t0, s_cur, false, flag);
+        fill_tile_params(sp, R, EnsTile(), s_t0, s_cur, false, flag);
     }
     __syncthreads();
     const uint32_t t0 = s_t0;
     const int cur = s_cur;
-    const bool unit = sp.unit != 0;   // every rate 1: the unit path
     const uint32_t gplane = (uint32_t)nx * ny;
-    const uint32_t n4 = (uint32_t)rows * nx / 4;   // float4 of a plane's own rows
+    const uint32_t n4 = P / 4;   // float4 of a plane's own rows
     {
         const float4 *src = reinterpret_cast<const float4 *>(R.buf[cur]);
         for (uint32_t k = threadIdx.x; k < 9 * n4; k += blockDim.x) {
@@ -204,42 +114,104 @@ ens_resident_kernel(const EnsRep *__restrict__ reps, const int *__restrict__ lis
                 __ldcg(src + (i * gplane + (uint32_t)ybase * nx) / 4 + e);
         }
     }
-    const int ncopy = (nb + 1) * (H + 1);
+    const int npair = (int)P / 2, lg = __ffs(nx) - 2;          // nx / 2 = 1 << lg
+    const uint32_t prev = (rank + C - 1) % C, next = (rank + 1) % C;
+    sync_all<C>();
     for (int s = 0; s < nsteps; ++s) {
-        sync_all<C>();   // the previous step's writes (or the load) are done
-        // the copied rows: the lower halo of band 0, then each band's upper halo
-        for (int c = band; c < ncopy; c += nb) {
-            int drow, from;
-            uint32_t srank = rank;
-            if (c <= H) {
-                drow = rows + c;
-                from = rows - (H + 1) + c;
-                srank = (rank + C - 1) % C;
-            } else {
-                const int b = c / (H + 1) - 1, j = c - (b + 1) * (H + 1);
-                drow = rows + (H + 1) * (1 + b) + j;
-                if (b < nb - 1) {
-                    from = (b + 1) * hb + j;
-                } else {
-                    from = j;
-                    srank = (rank + 1) % C;
-                }
-            }
-            const float *src = sm + from * nx + tx;
-            float *dst = sm + drow * nx + tx;
+        float *drho = (sample && s == nsteps - 1) ? R.drho : nullptr;
+        float2 q[NP][NQ];
 #pragma unroll
-            for (int i = 0; i < 9; ++i)
-                dst[i * P] = (C > 1 && srank != rank) ? ld_cluster(src + i * P, srank) : src[i * P];
+        for (int k = 0; k < NP; ++k) {
+            const int idx = threadIdx.x + k * blockDim.x;
+            if (idx >= npair) continue;
+            const int y = idx >> lg, x = 2 * (idx & (nx / 2 - 1));
+            const int xm = (x - 1) & (nx - 1), xq = (x + 2) & (nx - 1);
+            // element (row yy, column c) of plane i, -1 <= yy <= rows
+            auto ld = [&](int i, int yy, int c) {
+                const float *pl = sm + i * P + c;
+                if (C > 1 && yy < 0) return ld_cluster(pl + (rows - 1) * nx, prev);
+                if (C > 1 && yy >= rows) return ld_cluster(pl, next);
+                return pl[(yy < 0 ? rows - 1 : yy >= rows ? 0 : yy) * nx];
+            };
+            auto mid = [&](int i, int yy) {
+                if (C > 1 && (yy < 0 || yy >= rows))
+                    return make_float2(ld(i, yy, x), ld(i, yy, x + 1));
+                return *reinterpret_cast<const float2 *>(
+                    sm + i * P + (yy < 0 ? rows - 1 : yy >= rows ? 0 : yy) * nx + x);
+            };
+            auto plus = [&](int i, int yy) { return make_float2(ld(i, yy, xm), ld(i, yy, x)); };
+            auto minus = [&](int i, int yy) {
+                return make_float2(ld(i, yy, x + 1), ld(i, yy, xq));
+            };
+            const float2 g[9] = {mid(0, y),      plus(1, y),      mid(2, y - 1),
+                                 minus(3, y),    mid(4, y + 1),   plus(5, y - 1),
+                                 minus(6, y - 1), minus(7, y + 1), plus(8, y + 1)};
+            const float2 s9 = sum9(g);
+            const float2 d = delta_psi(s9, sp.psi_kind, sp.rho0, sp.psi_c, sp.psi_b);
+            // delta psi into row r of the CTA `to`, with the periodic columns
+            auto put = [&](int r, uint32_t to, bool remote) {
+                float *a = sa + (r + H) * W + 2, *b = sb + (r + H) * W + 3;
+                auto st = [&](float *q_, float v) {
+                    if (remote) st_cluster(q_, to, v);
+                    else *q_ = v;
+                };
+                st(a + x, d.x);
+                st(a + x + 1, d.y);
+                st(b + x, d.x);
+                st(b + x + 1, d.y);
+                if (x == 0) {
+                    st(a + nx, d.x);
+                    st(a + nx + 1, d.y);
+                    st(b + nx, d.x);
+                }
+                if (x == nx - 2) {
+                    st(a - 2, d.x);
+                    st(a - 1, d.y);
+                    st(b - 1, d.y);
+                }
+            };
+            put(y, rank, false);
+            if (y < H) put(rows + y, prev, C > 1);
+            if (y >= rows - H) put(y - rows, next, C > 1);
+            if constexpr (UNIT) {
+                unit_moments(g, q[k][0], q[k][1], q[k][2]);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 9; ++i) q[k][i] = g[i];
+            }
+            if (drho)
+                *reinterpret_cast<float2 *>(drho + (uint32_t)(ybase + y) * nx + x) = s9;
         }
-        if (threadIdx.x == 0) {
-            sp.step = t0 + (uint32_t)s;
-            sp.drho_out = (sample && s == nsteps - 1) ? R.drho : nullptr;
+        sync_all<C>();   // delta psi is complete and the old state has been read
+#pragma unroll
+        for (int k = 0; k < NP; ++k) {
+            const int idx = threadIdx.x + k * blockDim.x;
+            if (idx >= npair) continue;
+            const int y = idx >> lg, x = 2 * (idx & (nx / 2 - 1));
+            const float *a = sa + (y + H) * W + 2 + x, *b = sb + (y + H) * W + 2 + x;
+            auto at = [&](int ex, int ey) {
+                return *reinterpret_cast<const float2 *>(
+                    ex == 1 ? b + ey * W + 2 : ex == -1 ? b + ey * W : a + ey * W + ex);
+            };
+            float2 sx, sy;
+            force_sums<ORDER>(at, sx, sy);
+            const float2 pf = vmul(bc<float2>(sp.force_pref), vadd(bc<float2>(sp.psi0), at(0, 0)));
+            const float2 Fx = vmul(pf, sx), Fy = vmul(pf, sy);
+            float2 f[9];
+            const uint32_t site = (uint32_t)(ybase + y) * nx + x;
+            if constexpr (UNIT)
+                collide_unit_m(q[k][0], q[k][1], q[k][2], Fx, Fy, sp, keys.rk, site,
+                               t0 + (uint32_t)s, f);
+            else collide<float2>(q[k], Fx, Fy, sp, keys.rk, site, t0 + (uint32_t)s, f);
+            float *w = sm + y * nx + x;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) *reinterpret_cast<float2 *>(w + i * P) = f[i];
+            const float2 chk = vadd(f[1], f[5]);
+            if (!(fabsf(chk.x) <= 3.402823466e38f && fabsf(chk.y) <= 3.402823466e38f))
+                atomicOr(flag, LB_STEP_NONFINITE);
         }
-        sync_all<C>();   // the copies are done before any row is overwritten
-        if (unit) res_sweep<ORDER, true>(sp, keys.rk, sm, ring, P, nx, rows, band, hb, tx, ybase);
-        else res_sweep<ORDER, false>(sp, keys.rk, sm, ring, P, nx, rows, band, hb, tx, ybase);
+        sync_all<C>();   // the new state is complete
     }
-    __syncthreads();
     {
         float4 *dst = reinterpret_cast<float4 *>(R.buf[cur ^ (nsteps & 1)]);
         for (uint32_t k = threadIdx.x; k < 9 * n4; k += blockDim.x) {
@@ -250,41 +222,57 @@ ens_resident_kernel(const EnsRep *__restrict__ reps, const int *__restrict__ lis
     }
 }
 
+template <int ORDER, int C>
+const void *res_fn_u(bool unit) {
+    return unit ? (const void *)ens_resident_kernel<ORDER, C, true>
+                : (const void *)ens_resident_kernel<ORDER, C, false>;
+}
 template <int ORDER>
-const void *res_fn_o(int C) {
+const void *res_fn_o(int C, bool unit) {
     switch (C) {
-    case 1: return (const void *)ens_resident_kernel<ORDER, 1>;
-    case 2: return (const void *)ens_resident_kernel<ORDER, 2>;
-    case 4: return (const void *)ens_resident_kernel<ORDER, 4>;
-    case 8: return (const void *)ens_resident_kernel<ORDER, 8>;
+    case 1: return res_fn_u<ORDER, 1>(unit);
+    case 2: return res_fn_u<ORDER, 2>(unit);
+    case 4: return res_fn_u<ORDER, 4>(unit);
+    case 8: return res_fn_u<ORDER, 8>(unit);
     default: return nullptr;
     }
 }
-const void *res_fn(int stencil, int C) {
-    return stencil == 4 ? res_fn_o<4>(C) : stencil == 6 ? res_fn_o<6>(C) : res_fn_o<8>(C);
+const void *res_fn(int stencil, int C, bool unit) {
+    return stencil == 4   ? res_fn_o<4>(C, unit)
+           : stencil == 6 ? res_fn_o<6>(C, unit)
+                          : res_fn_o<8>(C, unit);
+}
+
+// Threads of a CTA of `rows` rows: a pair of sites each, as far as they go.
+int res_block(int nx, int rows, bool unit) {
+    const int pairs = rows * nx / 2;
+    return pairs < res_threads(unit) ? (pairs + 31) / 32 * 32 : res_threads(unit);
 }
 
 }  // namespace
 
-size_t resident_smem(int nx, int rows, int hb, int stencil) {
-    const int H = stencil == 4 ? 1 : 2, ring = H == 1 ? 4 : 8;
-    if ((nx != 32 && nx != 64 && nx != 128) || hb < 2 * H + 2 || rows % hb) return 0;
-    const int nb = rows / hb;
-    if (nb * nx > kResMaxThreads) return 0;
-    return ((size_t)9 * (rows + (nb + 1) * (H + 1)) * nx + (size_t)nb * ring * nx) *
-           sizeof(float);
+size_t resident_smem(int nx, int rows, int stencil) {
+    const int H = stencil == 4 ? 1 : 2;
+    if ((nx != 32 && nx != 64 && nx != 128) || rows < 8 || rows % 8 || rows * nx > kResMaxSites)
+        return 0;
+    return ((size_t)9 * rows * nx + (size_t)2 * (rows + 2 * H) * (nx + 4)) * sizeof(float);
 }
 
 cudaError_t resident_prepare(int stencil, int C, size_t smem) {
-    const void *fn = res_fn(stencil, C);
-    if (!fn) return cudaErrorInvalidValue;
-    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    for (bool unit : {false, true}) {
+        const void *fn = res_fn(stencil, C, unit);
+        if (!fn) return cudaErrorInvalidValue;
+        const cudaError_t e =
+            cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
-int resident_max_clusters(int stencil, int C, int nx, int rows, int hb, size_t smem) {
-    const void *fn = res_fn(stencil, C);
+int resident_max_clusters(int stencil, int C, int nx, int rows, bool unit, size_t smem) {
+    const void *fn = res_fn(stencil, C, unit);
     if (!fn) return 0;
-    const int threads = rows / hb * nx;
+    const int threads = res_block(nx, rows, unit);
     if (C == 1) {
         int n = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, threads, smem) != cudaSuccess)
@@ -308,13 +296,13 @@ int resident_max_clusters(int stencil, int C, int nx, int rows, int hb, size_t s
 }
 
 cudaError_t launch_ens_resident(const ResLaunch &a, cudaStream_t s) {
-    const void *fn = res_fn(a.stencil, a.C);
+    const void *fn = res_fn(a.stencil, a.C, a.unit);
     if (!fn || a.nres < 1) return cudaErrorInvalidValue;
     const int rows = a.ny / a.C;
-    const size_t smem = resident_smem(a.nx, rows, a.hb, a.stencil);
+    const size_t smem = resident_smem(a.nx, rows, a.stencil);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(a.nres * a.C);
-    cfg.blockDim = dim3(rows / a.hb * a.nx);
+    cfg.blockDim = dim3(res_block(a.nx, rows, a.unit));
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr;
@@ -329,9 +317,9 @@ cudaError_t launch_ens_resident(const ResLaunch &a, cudaStream_t s) {
     const EnsClock *clk = a.clk;
     int *flag = a.flag;
     const EnsKeys keys = a.keys;
-    int nsteps = a.nsteps, sample = a.sample, hb = a.hb;
-    void *args[] = {(void *)&reps, (void *)&list, (void *)&clk,    (void *)&flag,
-                    (void *)&keys, (void *)&nsteps, (void *)&sample, (void *)&hb};
+    int nsteps = a.nsteps, sample = a.sample;
+    void *args[] = {(void *)&reps, (void *)&list,   (void *)&clk,   (void *)&flag,
+                    (void *)&keys, (void *)&nsteps, (void *)&sample};
     return cudaLaunchKernelExC(&cfg, fn, args);
 }
 

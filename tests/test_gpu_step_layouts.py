@@ -82,3 +82,30 @@ def test_ensemble_bands_match_lattices(stencil, strip):
             assert np.array_equal(g.populations(), e.populations(r)), (launch, r)
             g.close()
         e.close()
+
+
+@pytest.mark.parametrize("stencil,tau", [(4, 1.0), (4, 0.9), (8, 1.0), (8, 0.9)])
+@pytest.mark.parametrize("nx,ny", [(32, 8), (32, 24), (64, 8), (64, 40), (128, 32), (128, 256)])
+def test_resident_shapes_match_tiles(nx, ny, stencil, tau):
+    """Fewer pairs than threads, a last round of pairs that some threads sit out, one
+    CTA and clusters of up to eight (128 x 256), windows ending in a sample."""
+    from paper_2212_07848_gb300 import abi
+    from paper_2212_07848_gb300.ensemble import Ensemble
+    reps = [(nx, ny, -4.0 - 0.1 * r, tau, 1e-5, 0.7) for r in range(3)]
+    out = []
+    for mode in (abi.LB_ENS_RESIDENT_ON, abi.LB_ENS_RESIDENT_OFF):
+        e = Ensemble(reps, stencil=stencil, seed=4)
+        e.set_resident(mode)
+        assert e.num_resident == (3 if mode == abi.LB_ENS_RESIDENT_ON else 0)
+        e.set_launch(abi.LB_ENS_PERSISTENT)
+        e.init(0.01)
+        pow2 = (ny & (ny - 1)) == 0
+        if pow2:
+            e.sk_config(4, 4)
+        e.step(1)
+        e.step(12)
+        e.sync()
+        out.append([e.populations(r) for r in range(3)] +
+                   ([e.structure_factor(r)[0] for r in range(3)] if pow2 else []))
+        e.close()
+    assert all(np.array_equal(a, b) for a, b in zip(*out))
