@@ -401,7 +401,7 @@ int lb3_init(lb3_ctx *h, double rho0, uint64_t seed, double init_amp);
  * LB_PSI_EXP); takes effect from the next step. */
 int lb3_set_psi(lb3_ctx *h, int psi_kind, double psi_p1, double psi_p2);
 int lb3_set_replica(lb3_ctx *h, uint32_t replica);
-/* z planes marched by one CTA (performance only). */
+/* z planes marched by one CTA (performance only; by default chosen from the box). */
 int lb3_set_strip(lb3_ctx *h, int planes);
 int lb3_step(lb3_ctx *h, int n);
 int lb3_sync(lb3_ctx *h);

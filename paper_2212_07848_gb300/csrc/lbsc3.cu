@@ -104,6 +104,10 @@ constexpr int kTX3 = 32;
 constexpr int kTYMin3 = 4;   // ny must be a multiple of this
 static_assert(kTX3 == 32, "one warp per interior row");
 template <int TY> constexpr int threads3() { return (kTX3 + 2) * (TY + 2); }
+// CTAs of the step kernel that an SM holds.
+template <typename T, int TY> constexpr int resident3() {
+    return sizeof(T) == 4 && TY == 4 ? 4 : 2;
+}
 
 // Thread -> (tx, ty) of the 34 x (TY + 2) block: warps 0 .. TY - 1 are the
 // interior rows (ty = 1 .. TY, tx = 1 .. 32); then the two ring rows
@@ -347,7 +351,7 @@ __device__ __forceinline__ void collide3_m(const T m[19], T Fx, T Fy, T Fz, cons
 
 
 template <typename T, bool SAMPLE, bool UNIT, int TY>
-__global__ void __launch_bounds__(threads3<TY>(), (sizeof(T) == 4 && TY == 4) ? 4 : 2)
+__global__ void __launch_bounds__(threads3<TY>(), resident3<T, TY>())
 step3_kernel(const K3<T> p) {
     constexpr int kBX3 = kTX3 + 2, kBY3 = TY + 2;
     __shared__ T s_psi[4][kBY3][kBX3];   // ring of planes: one barrier per plane suffices
@@ -904,7 +908,7 @@ struct lb3_ctx {
     long long sk_start = 0, sk_count = 0, t = 0;
     uint64_t seed = 0;
     uint32_t replica = 0;
-    int strip_z = 32;
+    int strip_z = 1;
     bool inited = false;
 };
 
@@ -958,27 +962,58 @@ template <typename T, int TY>
 int step3_launch(lb3_ctx *h, const K3<T> &k, bool sample) {
     const dim3 grid(h->nx / kTX3, h->ny / TY, (h->nz + h->strip_z - 1) / h->strip_z);
     const int nt = threads3<TY>();
-    bool done = false;
-    if constexpr (std::is_same<T, float>::value) {
-        if (h->tau == 1.0) {   // gamma = 0: the unit-relaxation path
-            if (sample) step3_kernel<T, true, true, TY><<<grid, nt, 0, h->stream>>>(k);
-            else step3_kernel<T, false, true, TY><<<grid, nt, 0, h->stream>>>(k);
-            done = true;
-        }
+    if (h->tau == 1.0) {   // gamma = 0: the unit-relaxation path
+        if (sample) step3_kernel<T, true, true, TY><<<grid, nt, 0, h->stream>>>(k);
+        else step3_kernel<T, false, true, TY><<<grid, nt, 0, h->stream>>>(k);
+    } else if (sample) {
+        step3_kernel<T, true, false, TY><<<grid, nt, 0, h->stream>>>(k);
+    } else {
+        step3_kernel<T, false, false, TY><<<grid, nt, 0, h->stream>>>(k);
     }
-    if (!done && sample) step3_kernel<T, true, false, TY><<<grid, nt, 0, h->stream>>>(k);
-    else if (!done) step3_kernel<T, false, false, TY><<<grid, nt, 0, h->stream>>>(k);
     L3_CHECK(cudaGetLastError());
     return LB_OK;
 }
+
+// Rows of the step kernel's tile.
+int tile_rows3(int ny, int precision) { return precision == LB_FP32 && ny % 8 == 0 ? 8 : 4; }
 
 template <typename T>
 int step3_once(lb3_ctx *h, bool sample) {
     const K3<T> k = params3<T>(h, sample);
     if constexpr (std::is_same<T, float>::value) {
-        if (h->ny % 8 == 0) return step3_launch<T, 8>(h, k, sample);
+        if (tile_rows3(h->ny, LB_FP32) == 8) return step3_launch<T, 8>(h, k, sample);
     }
     return step3_launch<T, 4>(h, k, sample);
+}
+
+// Planes per CTA when none is set.  A CTA pulls two planes more than it stores, so
+// on a box that fills the SMs many times over long strips win: 32 (256^3: 556 us a
+// step, 16 planes 564, 8 planes 602).  A box that 32 planes give to at most four
+// waves of CTAs takes the height whose waves cost the fewest plane times (s + 2 per
+// wave, the remainder strips in the slots left over), if that is 15% below 32
+// planes; nearer ones the count does not order (256 x 256 x 40: 38 against 44 counted,
+// 103 us against 97).  64^3 17.0 us against 51.9 with 32 planes, 96^3 38.0
+// against 60.0, 96 x 84 x 50 23.2 against 48.1, 192 x 128 x 160 133 against 165, FP64
+// 64^3 463 against 1059; 128^3 (84.6 us) keeps 32.
+int default_strip3(int nx, int ny, int nz, int precision, int sms) {
+    const int ty = tile_rows3(ny, precision);
+    const long long tiles = (long long)(nx / kTX3) * (ny / ty);
+    const long long slots =
+        (long long)sms * (precision == LB_FP32 && ty == 4 ? resident3<float, 4>()
+                                                          : resident3<float, 8>());
+    auto cost = [&](int s) {
+        const long long full = tiles * (nz / s), rem = nz % s;
+        const long long waves = (full + slots - 1) / slots;
+        long long left = rem ? tiles - (waves * slots - full) * ((s + 2) / (rem + 2)) : 0;
+        left = left > 0 ? (left + slots - 1) / slots : 0;
+        return waves * (s + 2) + left * (rem + 2);
+    };
+    const int long_strip = nz < 32 ? nz : 32;
+    if (tiles * ((nz + long_strip - 1) / long_strip) > 4 * slots) return long_strip;
+    int best = nz;
+    for (int s = nz - 1; s >= 1; --s)
+        if (cost(s) < cost(best)) best = s;
+    return 20 * cost(best) <= 17 * cost(long_strip) ? best : long_strip;
 }
 
 // Lines per block of a length-n transform: as many as fit 128 KB (at most 64).
@@ -1102,7 +1137,9 @@ int lb3_create(lb3_ctx **out, int nx, int ny, int nz, double G, double tau, doub
     h->precision = precision;
     h->esize = precision == LB_FP32 ? 4 : 8;
     h->n = (size_t)nx * ny * nz;
-    h->strip_z = nz < 32 ? nz : 32;
+    int sms = 1;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->dev);
+    h->strip_z = default_strip3(nx, ny, nz, precision, sms);
     if (stream) {
         h->stream = (cudaStream_t)stream;
     } else if (cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking) == cudaSuccess) {

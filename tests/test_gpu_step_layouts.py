@@ -109,3 +109,24 @@ def test_resident_shapes_match_tiles(nx, ny, stencil, tau):
                    ([e.structure_factor(r)[0] for r in range(3)] if pow2 else []))
         e.close()
     assert all(np.array_equal(a, b) for a, b in zip(*out))
+
+
+@pytest.mark.parametrize("nx,ny,nz,precision,tau", [
+    (32, 4, 3, "fp32", 1.0), (32, 32, 33, "fp32", 0.8), (96, 84, 50, "fp32", 1.0),
+    (64, 64, 64, "fp32", 1.0), (32, 8, 200, "fp32", 1.0), (32, 12, 9, "fp64", 1.0),
+    (64, 64, 20, "fp64", 0.8)])
+def test_3d_default_strip_agrees(nx, ny, nz, precision, tau):
+    """The default cut along z against one strip, single planes and a remainder."""
+    from paper_2212_07848_gb300.lattice3 import Lattice3
+    states = []
+    for strip in (0, nz, 1, 2):
+        g = Lattice3(nx, ny, nz, -3.6, tau, 1e-6, precision=precision)
+        if strip:
+            g.set_strip(strip)
+        g.init(0.7, 5, 0.02)
+        g.step(4)
+        states.append(g.populations())
+        g.close()
+    assert np.isfinite(states[0]).all()
+    for s in states[1:]:
+        assert np.array_equal(states[0], s)
