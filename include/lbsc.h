@@ -481,6 +481,20 @@ int lb_nn_relu_mask(const void *dy, const void *y, void *dz, size_t n, void *str
 int lb_nn_pool2(const void *x, void *y, int nb, int h, int w_, int c, int backward, void *stream);
 /* Nearest 2x upsampling of [nb][h][w][c] (backward: sum of the 2x2 block). */
 int lb_nn_up2(const void *x, void *y, int nb, int h, int w_, int c, int backward, void *stream);
+/* Chains of these passes on one read of their inputs, with the results of the
+ * single calls (BF16 roundings included).  c must be a multiple of 8 and every
+ * buffer 16-byte aligned (LB_ERR_ARG otherwise).
+ *   lb_nn_up2_relu_bwd: ds = backward up2 of dy [nb][2h][2w][c] (ds may be NULL),
+ *     dz = ds where act > 0, else 0 (ds, act, dz [nb][h][w][c]).
+ *   lb_nn_pool2_relu_bwd: t = backward pool2 of dy [nb][h/2][w/2][c], plus add
+ *     (may be NULL); dz = t where act > 0, else 0 (add, act, dz [nb][h][w][c]).
+ *   lb_nn_add_up2: s = a + b (s may be NULL), y = up2 of s [nb][2h][2w][c]. */
+int lb_nn_up2_relu_bwd(const void *dy, const void *act, void *ds, void *dz, int nb, int h, int w_,
+                       int c, void *stream);
+int lb_nn_pool2_relu_bwd(const void *dy, const void *add, const void *act, void *dz, int nb, int h,
+                         int w_, int c, void *stream);
+int lb_nn_add_up2(const void *a, const void *b, void *s, void *y, int nb, int h, int w_, int c,
+                  void *stream);
 /* y = a + b elementwise (n values). */
 int lb_nn_add(const void *a, const void *b, void *y, size_t n, void *stream);
 /* Coarse-grained density of a lattice state: FP32 out [ny/f][nx/f] = (mean of

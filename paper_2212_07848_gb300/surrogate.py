@@ -91,14 +91,13 @@ class SurrogateNet:
         z = lambda h, c: t.empty((nb, h, h, c), dtype=bf, device="cuda")
         self.nb = nb
         self.a1, self.p1, self.a2, self.p2 = z(n, 32), z(n // 2, 32), z(n // 2, 64), z(n // 4, 64)
-        self.a3, self.u3, self.a4, self.s4 = z(n // 4, 128), z(n // 2, 128), z(n // 2, 64), z(n // 2, 64)
+        self.a3, self.u3, self.a4 = z(n // 4, 128), z(n // 2, 128), z(n // 2, 64)
         self.u4, self.y = z(n, 64), z(n, 16)
         self.inc, self.dinc = (z(n, 1), z(n, 1)) if self.flux else (None, None)
         # gradients
         self.dy, self.du4, self.ds4, self.dz4 = z(n, 16), z(n, 64), z(n // 2, 64), z(n // 2, 64)
-        self.du3, self.da3, self.dz3, self.dp2 = z(n // 2, 128), z(n // 4, 128), z(n // 4, 128), z(n // 4, 64)
-        self.da2, self.dz2, self.dp1 = z(n // 2, 64), z(n // 2, 64), z(n // 2, 32)
-        self.da1, self.dz1, self.tmp2 = z(n, 32), z(n, 32), z(n // 2, 64)
+        self.du3, self.dz3, self.dp2 = z(n // 2, 128), z(n // 4, 128), z(n // 4, 64)
+        self.dz2, self.dp1, self.dz1 = z(n // 2, 64), z(n // 2, 32), z(n, 32)
         sizes = [n, n // 2, n // 4, n // 2, n]
         ws = max(self.L.lb_nn_wgrad_workspace(nb, h, h, ci, co)
                  for h, (ci, co) in zip(sizes, LAYERS))
@@ -120,8 +119,8 @@ class SurrogateNet:
         self._conv(self.p2, 2, self.a3, 1, n // 4)
         _check(L.lb_nn_up2(_p(self.a3), _p(self.u3), nb, n // 4, n // 4, 128, 0, self.s), "up")
         self._conv(self.u3, 3, self.a4, 1, n // 2)
-        _check(L.lb_nn_add(_p(self.a4), _p(self.a2), _p(self.s4), self.s4.numel(), self.s), "add")
-        _check(L.lb_nn_up2(_p(self.s4), _p(self.u4), nb, n // 2, n // 2, 64, 0, self.s), "up")
+        _check(L.lb_nn_add_up2(_p(self.a4), _p(self.a2), None, _p(self.u4), nb, n // 2, n // 2, 64,
+                               self.s), "add up")
         self._conv(self.u4, 4, self.y, 0, n)
         if self.flux:
             _check(L.lb_nn_flux_div(_p(self.y), _p(self.inc), 16, nb, n, n, 0, self.s), "flux")
@@ -190,21 +189,20 @@ class SurrogateNet:
             _p(dz), _p(self.wb[i]), None, _p(out), nb, h, h, LAYERS[i][1], LAYERS[i][0], 0, 1, s), "dgrad")
         wg(self.u4, self.dy, 4, n)
         dg(self.dy, 4, self.du4, n)
-        _check(L.lb_nn_up2(_p(self.du4), _p(self.ds4), nb, n // 2, n // 2, 64, 1, s), "upb")
-        _check(L.lb_nn_relu_mask(_p(self.ds4), _p(self.a4), _p(self.dz4), self.dz4.numel(), s), "relu")
+        _check(L.lb_nn_up2_relu_bwd(_p(self.du4), _p(self.a4), _p(self.ds4), _p(self.dz4), nb,
+                                    n // 2, n // 2, 64, s), "upb relu")
         wg(self.u3, self.dz4, 3, n // 2)
         dg(self.dz4, 3, self.du3, n // 2)
-        _check(L.lb_nn_up2(_p(self.du3), _p(self.da3), nb, n // 4, n // 4, 128, 1, s), "upb")
-        _check(L.lb_nn_relu_mask(_p(self.da3), _p(self.a3), _p(self.dz3), self.dz3.numel(), s), "relu")
+        _check(L.lb_nn_up2_relu_bwd(_p(self.du3), _p(self.a3), None, _p(self.dz3), nb, n // 4,
+                                    n // 4, 128, s), "upb relu")
         wg(self.p2, self.dz3, 2, n // 4)
         dg(self.dz3, 2, self.dp2, n // 4)
-        _check(L.lb_nn_pool2(_p(self.dp2), _p(self.tmp2), nb, n // 2, n // 2, 64, 1, s), "poolb")
-        _check(L.lb_nn_add(_p(self.tmp2), _p(self.ds4), _p(self.da2), self.da2.numel(), s), "add")
-        _check(L.lb_nn_relu_mask(_p(self.da2), _p(self.a2), _p(self.dz2), self.dz2.numel(), s), "relu")
+        _check(L.lb_nn_pool2_relu_bwd(_p(self.dp2), _p(self.ds4), _p(self.a2), _p(self.dz2), nb,
+                                      n // 2, n // 2, 64, s), "poolb relu")
         wg(self.p1, self.dz2, 1, n // 2)
         dg(self.dz2, 1, self.dp1, n // 2)
-        _check(L.lb_nn_pool2(_p(self.dp1), _p(self.da1), nb, n, n, 32, 1, s), "poolb")
-        _check(L.lb_nn_relu_mask(_p(self.da1), _p(self.a1), _p(self.dz1), self.dz1.numel(), s), "relu")
+        _check(L.lb_nn_pool2_relu_bwd(_p(self.dp1), None, _p(self.a1), _p(self.dz1), nb, n, n, 32,
+                                      s), "poolb relu")
         wg(x, self.dz1, 0, n)
         if dx is not None:
             dg(self.dz1, 0, dx, n)

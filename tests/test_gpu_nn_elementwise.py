@@ -105,3 +105,42 @@ def test_bias_and_weight_sums_add_up(cin, cout, h):
         ref = 2.0 * torch.einsum("bhwn,bhwc->nc", yd, s)
         assert (dw[tap].double() - ref).abs().max() < 1e-5 * ref.abs().max() * 10
     assert (db.double() - 2 * yd.sum((0, 1, 2))).abs().max() < 1e-5 * yd.abs().sum() / cout
+
+
+@pytest.mark.parametrize("nb,h,w,c", [(1, 1, 1, 8), (2, 3, 5, 24), (1, 70, 9, 64), (3, 2, 40, 32)])
+def test_chains_equal_the_single_calls(nb, h, w, c):
+    """The chained passes against the calls that they replace, bit for bit."""
+    from paper_2212_07848_gb300 import abi
+    L = abi.load()
+    small, big = (nb, h, w, c), (nb, 2 * h, 2 * w, c)
+    sa, sb, fa, fb, act, facts = (_bf(s, i) for i, s in enumerate((small, small, big, big, small, big)))
+    act[:, :, ::2] = 0.0
+    new = lambda t: torch.full_like(t, 7.0)
+    n, m = sa.numel(), fa.numel()
+    # gradient of the upsampling, then the mask
+    s, z, s2, z2 = (new(sa) for _ in range(4))
+    assert L.lb_nn_up2(_p(fa), _p(s), nb, h, w, c, 1, None) == 0
+    assert L.lb_nn_relu_mask(_p(s), _p(act), _p(z), n, None) == 0
+    assert L.lb_nn_up2_relu_bwd(_p(fa), _p(act), _p(s2), _p(z2), nb, h, w, c, None) == 0
+    assert torch.equal(s2, s) and torch.equal(z2, z)
+    assert L.lb_nn_up2_relu_bwd(_p(fa), _p(act), None, _p(s2), nb, h, w, c, None) == 0
+    assert torch.equal(s2, z)
+    # gradient of the pooling, with and without a second branch, then the mask
+    t, f, f2 = (new(fa) for _ in range(3))
+    assert L.lb_nn_pool2(_p(sa), _p(t), nb, 2 * h, 2 * w, c, 1, None) == 0
+    for add in (None, fb):
+        if add is not None:
+            assert L.lb_nn_add(_p(t), _p(add), _p(t), m, None) == 0
+        assert L.lb_nn_relu_mask(_p(t), _p(facts), _p(f), m, None) == 0
+        assert L.lb_nn_pool2_relu_bwd(_p(sa), None if add is None else _p(add), _p(facts), _p(f2),
+                                      nb, 2 * h, 2 * w, c, None) == 0
+        assert torch.equal(f2, f)
+    # sum, then the upsampling
+    assert L.lb_nn_add(_p(sa), _p(sb), _p(s), n, None) == 0
+    assert L.lb_nn_up2(_p(s), _p(f), nb, h, w, c, 0, None) == 0
+    assert L.lb_nn_add_up2(_p(sa), _p(sb), _p(s2), _p(f2), nb, h, w, c, None) == 0
+    assert torch.equal(s2, s) and torch.equal(f2, f)
+    # refused: channel counts and buffers off the 16-byte grid
+    off = _bf(big, 9, 1)
+    assert L.lb_nn_up2_relu_bwd(_p(fa), _p(act), None, _p(s2), nb, h, w, c - 4, None) != 0
+    assert L.lb_nn_add_up2(_p(sa), _p(sb), None, _p(off), nb, h, w, c, None) != 0
