@@ -200,6 +200,19 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t r[32]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// Zeros in N columns (16 or 32) of this warp's 32 lanes.
+template <int N> __device__ __forceinline__ void tmem_zero(uint32_t taddr) {
+    static_assert(N == 16 || N == 32, "columns");
+#pragma unroll
+    for (int c = 0; c < N; c += 16)
+        asm volatile(
+            "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, "
+            "%1, %1, %1, %1, %1, %1};" ::"r"(taddr + c),
+            "r"(0u)
+            : "memory");
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
+
 __device__ __forceinline__ void cp_async_commit() {
     asm volatile("cp.async.commit_group;\n" ::: "memory");
 }
@@ -363,9 +376,9 @@ cudaError_t launch_tc(const bf16 *x, const bf16 *w, const float *bias, bf16 *y, 
 }
 
 // ---------------------------------------------------------------------------
-// Persistent, warp-specialised variant.  One CTA per SM (192 threads):
+// Persistent, warp-specialised variant, one or more CTAs per SM (192 threads):
 //   warp 4  producer: stages the nine taps' weights of the CTA's output-channel
-//           block once, then input rows into a ring of R slots (cp.async,
+//           block once, then input rows into a ring of R slots (TMA,
 //           completion tracked on mbarriers), as far ahead as free slots allow;
 //   warp 5  MMA issuer (one thread): for each output row (128 pixels of one
 //           image row) the 9 x CIN/16 tcgen05.mma of its three input rows
@@ -375,13 +388,20 @@ cudaError_t launch_tc(const bf16 *x, const bf16 *w, const float *bias, bf16 *y, 
 //   warps 0-3 epilogue: tcgen05.ld of the accumulator (warp w owns lanes
 //           32w .. 32w+31 = pixels), bias, ReLU, BF16 stores, then release
 //           the accumulator.
+// An MMA of 16 to 64 columns is bound by the reads of its 128-row operand, which
+// that order makes three times.  Folded, each input row is read once: its 3 x CIN/16
+// MMAs of 3 BN columns go to the three output rows that it belongs to, neighbours in
+// a ring of accumulators.  An output's products are added in the same order, so the
+// results are the same bits.  8 x 256^2, 128 -> 64: 154 us in the first order (input
+// staged once per 32 channels), 74 us folded; 8 x 512^2, 64 -> 16: 180 and 84 us.
 // A CTA walks runs of consecutive output rows down a 128-pixel column band,
 // so each input row is staged once per run.  DG: the input gradient of a
 // forward layer (weights read transposed, taps mirrored), so the same kernel
 // serves forward and backward.  Every wait is bounded; a timeout stops every
 // role, and tensor memory is freed only after the committed MMAs finished.
 // ---------------------------------------------------------------------------
-template <int BN, int CIN>
+// FOLD: one MMA of N = 3 BN columns takes an input row to its three output rows.
+template <int BN, int CIN, bool FOLD>
 struct PCfg {
     // Input channels are staged in blocks of BC = min(CIN, 64) channels, one
     // TMA box each, whose pixel rows of SP = 2 BC bytes carry the matching
@@ -397,16 +417,28 @@ struct PCfg {
     static constexpr int ROW_BYTES = KB * 144 * SP;
     static constexpr int TAP_BYTES = BN * CIN * 2;
     static constexpr int B_BYTES = 9 * TAP_BYTES;
+    static_assert(!FOLD || 3 * BN <= 256, "N of an MMA");
+    // ring slots: a folded row is read once and needs no neighbours, so a short
+    // ring leaves room for a second CTA where that fits
     static constexpr int R0 = (220 * 1024 - B_BYTES) / ROW_BYTES;
-    static constexpr int R = R0 < 4 ? 4 : (R0 > 8 ? 8 : R0);   // ring slots
+    static constexpr int R1 = (110 * 1024 - B_BYTES) / ROW_BYTES;
+    static constexpr int R = !FOLD ? (R0 < 4 ? 4 : (R0 > 8 ? 8 : R0))
+                                   : (R1 >= 3 ? (R1 > 8 ? 8 : R1) : (R0 > 8 ? 8 : R0));
+    static constexpr int NACC = !FOLD ? 2 : (R1 >= 3 ? 256 : 512) / BN > 16 ? 16
+                                          : (R1 >= 3 ? 256 : 512) / BN;   // accumulators
     static constexpr int A_BYTES = R * ROW_BYTES;
     static constexpr int SMEM = A_BYTES + B_BYTES;
-    // B per tap: channel block kb of output channel n at kb * BN * SP + n * SP
-    // (16-byte chunks swizzled as TMA writes them)
-    static constexpr uint32_t LBO_B = BN * SP;
+    // B: channel block kb of output channel n of a tap at kb * LBO_B + n * SP from
+    // tap_off(tap) (16-byte chunks swizzled as TMA writes them).  FOLD: the taps of
+    // one dx are one operand of 3 BN rows, dy = 2 first.
+    static constexpr uint32_t LBO_B = (FOLD ? 3 : 1) * BN * SP;
+    __host__ __device__ static constexpr uint32_t tap_off(int tap) {
+        return FOLD ? (tap % 3) * 3 * TAP_BYTES + (2 - tap / 3) * BN * SP : tap * TAP_BYTES;
+    }
     static constexpr uint32_t ROW_TX = (uint32_t)CIN * 144 * 2;   // bytes landing per row
     static constexpr int ALIGN = 1024;                            // staging alignment
-    static constexpr uint32_t NCOLS = 2 * BN <= 32 ? 32 : (2 * BN <= 64 ? 64 : (2 * BN <= 128 ? 128 : 256));
+    static constexpr uint32_t NCOLS = NACC * BN;
+    static_assert(R >= 2 && NACC * BN >= 32 && NACC * BN <= 512, "plan");
 };
 constexpr int kTcpThreads = 192;
 
@@ -443,19 +475,20 @@ __device__ __forceinline__ bool mbar_wait_ab(uint64_t *bar, uint32_t parity, uin
 // (tm_xh: 8 channels x 8 pixels, the halo copies); tm_w: the weights as
 // [9][Cout][CIN] with a box of 8 channels x BN output channels (forward only;
 // the input gradient transposes the weights while staging them).
-template <int BN, int CIN, bool DG>
+template <int BN, int CIN, bool DG, bool FOLD>
 __global__ void __launch_bounds__(kTcpThreads, 1)
 conv3x3_tcp_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_xh,
                    const __grid_constant__ CUtensorMap tm_w, const bf16 *__restrict__ w,
                    const float *__restrict__ bias, bf16 *__restrict__ y, int nb, int H, int W,
                    int Cout, int relu, int ctas_per_block, int units_per_cta) {
-    using C = PCfg<BN, CIN>;
+    using C = PCfg<BN, CIN, FOLD>;
     constexpr int R = C::R;
     extern __shared__ __align__(128) uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t full[R], slot_free[R], acc_full[2], acc_empty[2], wfull;
+    __shared__ __align__(8) uint64_t full[R], slot_free[R], acc_full[C::NACC],
+        acc_empty[C::NACC], wfull;
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort, s_drained;
-    __shared__ float s_bias[BN];
+    __shared__ __align__(16) float s_bias[BN];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // aligned base for the bulk copies (128 bytes, 1024 for the swizzled
     // layout; the launch adds that much slack)
@@ -478,24 +511,31 @@ conv3x3_tcp_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     for (int i = tid; i < BN; i += kTcpThreads) s_bias[i] = bias ? bias[n0 + i] : 0.f;
     if (DG) {
         // w holds the forward layer's [9][CIN][Cout]; B[n][c] = w[8 - tap][c][n0 + n],
-        // staged by every thread (16-byte loads of 8 n, scattered 2-byte stores)
-        for (int v = tid; v < 9 * CIN * (BN / 8); v += kTcpThreads) {
-            const int tap = v / (CIN * (BN / 8)), rem = v - tap * (CIN * (BN / 8));
-            const int c = rem / (BN / 8), nc = rem - c * (BN / 8);
-            const uint4 q = *reinterpret_cast<const uint4 *>(
-                w + ((size_t)(8 - tap) * CIN + c) * Cout + n0 + nc * 8);
-            const bf16 *e = reinterpret_cast<const bf16 *>(&q);
+        // staged by every thread: two channels c, c + 1 of eight n (16-byte loads),
+        // stored as eight words.  Neighbouring lanes take neighbouring channel pairs,
+        // so a warp's store covers whole pixel rows and no bank twice (lanes along n
+        // and single 2-byte stores, 8 ways: 78 us against 65 at 8 x 256^2, 64 -> 128).
+        constexpr int CP = CIN / 2;
+#pragma unroll 4
+        for (int v = tid; v < 9 * CP * (BN / 8); v += kTcpThreads) {
+            const int tap = v / (CP * (BN / 8)), rem = v - tap * (CP * (BN / 8));
+            const int nc = rem / CP, c = 2 * (rem - nc * CP);
+            const bf16 *src = w + ((size_t)(8 - tap) * CIN + c) * Cout + n0 + nc * 8;
+            const uint4 q0 = *reinterpret_cast<const uint4 *>(src);
+            const uint4 q1 = *reinterpret_cast<const uint4 *>(src + Cout);
+            const uint32_t e0[4] = {q0.x, q0.y, q0.z, q0.w}, e1[4] = {q1.x, q1.y, q1.z, q1.w};
             // row n = nc * 8 + j of block c / BC; its 16-byte chunk ch = (c % BC) / 8
             // sits at chunk index ch ^ sw(n), the swizzle of an SP-byte row
             // (128: n % 8; 64: (n / 2) % 4; 32: (n / 4) % 2)
-            uint8_t *d = sB + tap * C::TAP_BYTES + (c / C::BC) * C::LBO_B + nc * 8 * C::SP +
+            uint8_t *d = sB + C::tap_off(tap) + (c / C::BC) * C::LBO_B + nc * 8 * C::SP +
                          (c & 7) * 2;
             const int ch = (c % C::BC) >> 3;
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const int n = nc * 8 + j;
                 const int sw = C::SP == 128 ? (n & 7) : (C::SP == 64 ? ((n >> 1) & 3) : ((n >> 2) & 1));
-                *reinterpret_cast<bf16 *>(d + j * C::SP + ((ch ^ sw) << 4)) = e[j];
+                *reinterpret_cast<uint32_t *>(d + j * C::SP + ((ch ^ sw) << 4)) =
+                    __byte_perm(e0[j / 2], e1[j / 2], j % 2 ? 0x7632 : 0x5410);
             }
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -505,7 +545,7 @@ conv3x3_tcp_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
             mbar_init(&full[i], 1);
             mbar_init(&slot_free[i], 1);
         }
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < C::NACC; ++i) {
             mbar_init(&acc_full[i], 1);
             mbar_init(&acc_empty[i], 4);
         }
@@ -538,7 +578,7 @@ conv3x3_tcp_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
                 constexpr int NBLK = C::KB, BCH = C::BC;      // boxes per tap, channels per box
                 for (int tap = 0; tap < 9; ++tap)
                     for (int kc = 0; kc < NBLK; ++kc)
-                        tma_load3(sB + tap * C::TAP_BYTES + kc * C::LBO_B, &tm_w, kc * BCH, n0, tap,
+                        tma_load3(sB + C::tap_off(tap) + kc * C::LBO_B, &tm_w, kc * BCH, n0, tap,
                                   &wfull);
             }
             for (long u = u_begin; u < u_end && !*abort;) {
@@ -595,8 +635,64 @@ conv3x3_tcp_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
             const uint32_t a_lo = desc_sw_lo(smem_u32(sA) + C::COL0);
             const uint32_t b_lo = desc_sw_lo(smem_u32(sB));
             if (!DG) ok = mbar_wait_ab(&wfull, 0, limit, abort);
+            if constexpr (FOLD) {
+                // input row q of a run goes to the output rows q - 2, q - 1, q (taps
+                // dy = 2, 1, 0): neighbouring accumulators of the ring and
+                // neighbouring rows of B, one MMA per K step (two where the ring
+                // wraps).  Accumulators come zeroed from the epilogue.  MMAs on
+                // overlapping accumulators of different start or width have no
+                // order of their own, so a row waits for such a one before it.
+                int g0 = 0;    // output rows of the runs before
+                int c0_last = -1, cnt_last = 0;
+                for (long u = u_begin; u < u_end && ok;) {
+                    int b, x0, row0, len;
+                    run_at(u, b, x0, row0, len);
+                    for (int q = 0; q < len + 2; ++q) {
+                        const int slot = nfree % R, g = g0 + q;
+                        ok = mbar_wait_ab(&full[slot], (uint32_t)((nfree / R) & 1), limit, abort);
+                        if (ok && q < len)
+                            ok = mbar_wait_ab(&acc_empty[g % C::NACC], (uint32_t)((g / C::NACC) & 1),
+                                              limit, abort);
+                        const int lo = q < 2 ? 0 : q - 2, cnt = min(q, len - 1) - lo + 1;
+                        const int c0 = (g0 + lo) % C::NACC;
+                        if (ok && nfree > 0 && (c0 != c0_last || cnt != cnt_last))
+                            ok = mbar_wait_ab(&slot_free[(nfree - 1) % R],
+                                              (uint32_t)(((nfree - 1) / R) & 1), limit, abort);
+                        if (!ok) break;
+                        tc_fence_after();
+                        c0_last = c0;
+                        cnt_last = cnt;
+                        const int n1 = min(cnt, C::NACC - c0), n2 = cnt - n1;
+                        const uint32_t d1 = tmem + (uint32_t)(c0 * BN);
+                        const uint32_t i1 = idesc_bf16(128, n1 * BN), i2 = idesc_bf16(128, n2 * BN);
+                        const uint32_t arow = a_lo + (uint32_t)slot * ((uint32_t)C::ROW_BYTES >> 4);
+                        const uint32_t b1 = b_lo + ((uint32_t)((lo - q + 2) * BN * C::SP) >> 4);
+                        const uint32_t b2 = b1 + ((uint32_t)(n1 * BN * C::SP) >> 4);
+#pragma unroll
+                        for (int dx = 0; dx < 3; ++dx) {
+#pragma unroll
+                            for (int j = 0; j < CIN / 16; ++j) {
+                                const uint32_t oa =
+                                    (uint32_t)(dx * C::SP + (j / C::KS) * C::LBO_A + (j % C::KS) * 32) >> 4;
+                                const uint32_t ob = (uint32_t)(dx * 3 * C::TAP_BYTES +
+                                                               (j / C::KS) * C::LBO_B + (j % C::KS) * 32) >> 4;
+                                tc_mma_lo(d1, arow + oa, DHI, b1 + ob, DHI, i1, 1u);
+                                if (n2) tc_mma_lo(tmem, arow + oa, DHI, b2 + ob, DHI, i2, 1u);
+                            }
+                        }
+                        tc_commit(&slot_free[slot]);
+                        ++nfree;
+                        if (q >= 2) {
+                            tc_commit(&acc_full[(g - 2) % C::NACC]);
+                            ++t;
+                        }
+                    }
+                    g0 += len;
+                    u += len;
+                }
+            }
             int seq0 = 0;
-            for (long u = u_begin; u < u_end && ok;) {
+            for (long u = u_begin; !FOLD && u < u_end && ok;) {
                 int b, x0, row0, len;
                 run_at(u, b, x0, row0, len);
                 for (int tt = 0; tt < len && ok; ++tt, ++t) {
@@ -663,8 +759,9 @@ conv3x3_tcp_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
             // this thread committed to.  The slot releases went to input rows
             // 0 .. nfree - 1 in order, so slot i took (nfree - 1 - i) / R + 1.
             bool drained = true;
-            for (int g = t > 2 ? t - 2 : 0; g < t; ++g)
-                drained = mbar_wait(&acc_full[g & 1], (uint32_t)((g >> 1) & 1), kTcWaitNs) && drained;
+            for (int g = t > C::NACC ? t - C::NACC : 0; g < t; ++g)
+                drained = mbar_wait(&acc_full[g % C::NACC], (uint32_t)((g / C::NACC) & 1), kTcWaitNs) &&
+                          drained;
             for (int i = 0; i < R && i < nfree; ++i) {
                 const int n = (nfree - 1 - i) / R + 1;
                 drained = mbar_wait(&slot_free[i], (uint32_t)((n - 1) & 1), kTcWaitNs) && drained;
@@ -677,26 +774,45 @@ conv3x3_tcp_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
         __syncwarp();
     } else {
         // ---------------- epilogue (warps 0-3) ----------------
-        long t = 0;
+        constexpr int CH = BN < 32 ? BN : 32;   // columns per tensor-memory access
+        int t = 0;
+        if (FOLD) {
+            const int used = (int)min((long)C::NACC, u_end - u_begin);
+            for (int i = 0; i < used; ++i) {
+#pragma unroll
+                for (int col = 0; col < BN; col += CH)
+                    tmem_zero<CH>(tmem + ((uint32_t)(warp * 32) << 16) + i * BN + col);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&acc_empty[i]);
+            }
+        }
         for (long u = u_begin; u < u_end && !*abort;) {
             int b, x0, row0, len;
             run_at(u, b, x0, row0, len);
             for (int tt = 0; tt < len; ++tt, ++t) {
-                if (!mbar_wait_ab(&acc_full[t & 1], (uint32_t)((t >> 1) & 1), limit, abort)) {
+                if (!mbar_wait_ab(&acc_full[t % C::NACC], (uint32_t)((t / C::NACC) & 1), limit, abort)) {
                     *abort = 1;
                     break;
                 }
                 tc_fence_after();
                 const uint32_t lane_base =
-                    tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)((t & 1) * BN);
-                bf16 *yout = y + (((size_t)b * H + row0 + tt) * W + x0 + warp * 32 + lane) * Cout + n0;
-                constexpr int CH = BN < 32 ? BN : 32;   // columns per tensor-memory load
+                    tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)((t % C::NACC) * BN);
+                constexpr int NQ = CH / 8;   // 16-byte pieces of a pixel's CH channels
+                // lanes that store one pixel's run together: one lane's 16-byte pieces
+                // lie in 32 lines at 64 channels (8 x 512^2, 16 -> 64: 70 us against 114;
+                // 16 -> 32: 53.2 against 55.6; folded 32 -> 32 26.7 without, 28.7 with)
+                constexpr int TR = BN >= 64 || !FOLD ? NQ : 1;
+                const int sub = lane & (TR - 1);
+                bf16 *yout = y + (((size_t)b * H + row0 + tt) * W + x0 + warp * 32 + lane - sub) * Cout +
+                             n0 + sub * 8;
 #pragma unroll
                 for (int col = 0; col < BN; col += CH) {
                     uint32_t rr[CH];
                     if constexpr (CH == 32) tmem_ld32(lane_base + col, rr);
                     else tmem_ld16(lane_base + col, rr);
-                    uint32_t packed[CH / 2];
+                    if (FOLD) tmem_zero<CH>(lane_base + col);
+                    uint32_t pk[NQ][4];
 #pragma unroll
                     for (int q = 0; q < CH / 2; ++q) {
                         float v0 = __uint_as_float(rr[2 * q]) + s_bias[col + 2 * q];
@@ -706,17 +822,33 @@ conv3x3_tcp_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
                             v1 = fmaxf(v1, 0.f);
                         }
                         __nv_bfloat162 h2 = __floats2bfloat162_rn(v0, v1);
-                        packed[q] = *reinterpret_cast<uint32_t *>(&h2);
+                        pk[q / 4][q % 4] = *reinterpret_cast<uint32_t *>(&h2);
                     }
-                    uint4 *dst = reinterpret_cast<uint4 *>(yout + col);
+                    // transpose pieces over TR lanes: piece q of this lane's pixel
+                    // becomes piece `sub` of pixel q
 #pragma unroll
-                    for (int q = 0; q < CH / 8; ++q)
-                        dst[q] = make_uint4(packed[4 * q], packed[4 * q + 1], packed[4 * q + 2],
-                                            packed[4 * q + 3]);
+                    for (int m = 1; m < TR; m <<= 1) {
+                        const bool up = lane & m;
+#pragma unroll
+                        for (int q = 0; q < NQ; ++q) {
+                            if (q & m) continue;
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                const uint32_t got =
+                                    __shfl_xor_sync(0xffffffffu, up ? pk[q][k] : pk[q | m][k], m);
+                                if (up) pk[q][k] = got;
+                                else pk[q | m][k] = got;
+                            }
+                        }
+                    }
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q)
+                        *reinterpret_cast<uint4 *>(yout + col + (TR > 1 ? q * Cout : q * 8)) =
+                            make_uint4(pk[q][0], pk[q][1], pk[q][2], pk[q][3]);
                 }
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&acc_empty[t & 1]);
+                if (lane == 0) mbar_arrive(&acc_empty[t % C::NACC]);
             }
             if (*abort) break;
             u += len;
@@ -779,10 +911,10 @@ bool tcp_map_span(CUtensorMap *m, const void *base, uint64_t d0, uint64_t d1, ui
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int BN, int CIN, bool DG>
+template <int BN, int CIN, bool DG, bool FOLD = false>
 cudaError_t launch_tcp(const bf16 *x, const bf16 *w, const float *bias, bf16 *y, int nb, int h,
                        int wd, int cout, int relu, cudaStream_t s) {
-    using C = PCfg<BN, CIN>;
+    using C = PCfg<BN, CIN, FOLD>;
     static_assert(C::SMEM + C::ALIGN <= 226 * 1024, "shared-memory plan too large");
     // at most 512 / NCOLS CTAs may share an SM's 512 tensor-memory columns:
     // the shared-memory request is padded so that no more fit
@@ -819,9 +951,9 @@ cudaError_t launch_tcp(const bf16 *x, const bf16 *w, const float *bias, bf16 *y,
         if (e == cudaSuccess)
             e = cudaDeviceGetAttribute(&regs_sm, cudaDevAttrMaxRegistersPerMultiprocessor, dev);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(conv3x3_tcp_kernel<BN, CIN, DG>,
+            e = cudaFuncSetAttribute(conv3x3_tcp_kernel<BN, CIN, DG, FOLD>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-        if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, conv3x3_tcp_kernel<BN, CIN, DG>);
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, conv3x3_tcp_kernel<BN, CIN, DG, FOLD>);
         if (e != cudaSuccess) {
             nsm = 0;
             return e;
@@ -834,36 +966,61 @@ cudaError_t launch_tcp(const bf16 *x, const bf16 *w, const float *bias, bf16 *y,
     int per_blk = std::max(1, nsm * per_sm / nblk);
     if (per_blk > units) per_blk = (int)units;
     const int per = (int)((units + per_blk - 1) / per_blk);
-    conv3x3_tcp_kernel<BN, CIN, DG><<<nblk * per_blk, kTcpThreads, kSmem, s>>>(
+    conv3x3_tcp_kernel<BN, CIN, DG, FOLD><<<nblk * per_blk, kTcpThreads, kSmem, s>>>(
         mx, mxh, mw, w, bias, y, nb, h, wd, cout, relu, per_blk, per);
     return cudaGetLastError();
 }
 
-// Channel block per CTA: all of cout where the weights and the ring fit,
-// else 32 (128 input channels).
+// Channel block per CTA: all of cout where the weights and the ring fit, else 64
+// (folded) or 32 (128 input channels).  Folded or not, by rows of 128 pixels per SM:
+// folding reads the input operand once instead of three times, which is what bounds
+// an MMA this narrow, and pays with two more rows a run and a wait per row.
+//   64 -> 16, 32: two folded CTAs share an SM and cover the waits: from 3 rows on
+//     (64 -> 16, 6.7 rows: 18.4 against 22.5 us; 108 rows: 84 against 180; 1 row 12.3
+//     against 10.2).
+//   128 -> 64: unfolded, the input is read once per 32 channels: from 3 rows on
+//     (3.4 rows: 22.5 against 29.7 us; 27 rows: 74 against 154), the input gradient
+//     41 against 55 us at 6.7 rows.
+//   the others from 16 rows on (64 -> 64, 27 rows: 49 against 55 us, 6.7 rows 24.6
+//     against 22.6; 128 -> 32, 6.7 rows 32.8 against 31.7; 32 -> 32, 27 rows: 26.7 against 29.2).
+//   16 channels: never (three MMAs a row; 16 -> 16 50 against 45 us at 108 rows).
 template <bool DG>
 cudaError_t launch_tcp_shape(const bf16 *x, const bf16 *w, const float *bias, bf16 *y, int nb,
                              int h, int wd, int cin, int cout, int relu, cudaStream_t s) {
+    static int nsm = 0;
+    if (!nsm) {
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
+    }
+    const long units = (long)nb * h * (wd / 128);
+    const bool few = units < 3l * nsm, many = units >= 16l * nsm;
 #define TCP(BN, CIN) return launch_tcp<BN, CIN, DG>(x, w, bias, y, nb, h, wd, cout, relu, s)
+#define TCP_FOLD(BN, CIN, WHEN)                                                                  \
+    if (WHEN) return launch_tcp<BN, CIN, DG, true>(x, w, bias, y, nb, h, wd, cout, relu, s)
     if (cin == 16) {
         if (cout == 16) TCP(16, 16);
         if (cout == 32) TCP(32, 16);
         if (cout == 64) TCP(64, 16);
         if (cout == 128) TCP(128, 16);
     } else if (cin == 32) {
-        if (cout == 16) TCP(16, 32);
-        if (cout == 32) TCP(32, 32);
-        if (cout == 64) TCP(64, 32);
+        if (cout == 16) { TCP_FOLD(16, 32, many); TCP(16, 32); }
+        if (cout == 32) { TCP_FOLD(32, 32, many); TCP(32, 32); }
+        if (cout == 64) { TCP_FOLD(64, 32, many); TCP(64, 32); }
         if (cout == 128) TCP(128, 32);
     } else if (cin == 64) {
-        if (cout == 16) TCP(16, 64);
-        if (cout == 32) TCP(32, 64);
-        if (cout == 64) TCP(64, 64);
+        if (cout == 16) { TCP_FOLD(16, 64, !few); TCP(16, 64); }
+        if (cout == 32) { TCP_FOLD(32, 64, !few); TCP(32, 64); }
+        if (cout == 64) { TCP_FOLD(64, 64, many); TCP(64, 64); }
         if (cout == 128) TCP(128, 64);
     } else if (cin == 128) {
-        if (cout == 16) TCP(16, 128);
+        if (cout == 16) { TCP_FOLD(16, 128, many); TCP(16, 128); }
+        if (cout % 64 == 0) TCP_FOLD(64, 128, !few);
+        if (cout == 32) TCP_FOLD(32, 128, many);
         if (cout % 32 == 0) TCP(32, 128);
     }
+#undef TCP_FOLD
 #undef TCP
     return cudaErrorNotSupported;
 }
