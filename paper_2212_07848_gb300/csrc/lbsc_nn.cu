@@ -280,25 +280,44 @@ wgrad_kernel(const bf16 *__restrict__ x, const bf16 *__restrict__ dy, float *__r
             }
 }
 
-// dw[i] += sum over chunks of part[chunk][i]: 32 weights to a block, its eight
-// warps sum every eighth chunk and are added in order (a fixed order).  Bound by
-// the partial sums' bytes where there are many weights (64 -> 128: 83 MB, 10.9 us,
-// 13.9 before) and by the chain of loads where there are few: one thread per weight
-// over all chunks left 18 blocks for 16 -> 32 (33.6 us; 8.6 us now).
+// dw[i] += sum over chunks of part[chunk][i]: a block's eight warps sum every eighth
+// chunk of its 32 V weights and are added in order (a fixed order).  Bound by the
+// partial sums' bytes where there are many weights: then V = 4, a 16-byte load per
+// chunk (64 -> 128: 83 MB in 8.6 us; V = 1 10.6; one thread per weight 13.9.
+// 128 -> 128: 29 MB in 8.9 us; V = 1 18.4).  Where there are few, by the chain of
+// loads: one thread per weight over all chunks left 18 blocks for 16 -> 32 (33.6 us;
+// V = 1 8.6 us).
 constexpr int kRedWarps = 8;
+template <int V>
 __global__ void __launch_bounds__(32 * kRedWarps)
 wgrad_reduce_kernel(const float *__restrict__ part, float *__restrict__ dw, size_t n, int nchunk) {
-    __shared__ float sh[kRedWarps][32];
+    __shared__ float sh[kRedWarps][32 * V];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const size_t i = (size_t)blockIdx.x * 32 + lane;   // n is a multiple of 32
-    float s = 0.f;
+    const size_t i = ((size_t)blockIdx.x * 32 + lane) * V;   // n is a multiple of 128
+    float s[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) s[v] = 0.f;
 #pragma unroll 8
-    for (int ch = w; ch < nchunk; ch += kRedWarps) s += part[(size_t)ch * n + i];
-    sh[w][lane] = s;
+    for (int ch = w; ch < nchunk; ch += kRedWarps) {
+        if constexpr (V == 4) {
+            const float4 q = *reinterpret_cast<const float4 *>(part + (size_t)ch * n + i);
+            s[0] += q.x;
+            s[1] += q.y;
+            s[2] += q.z;
+            s[3] += q.w;
+        } else {
+            s[0] += part[(size_t)ch * n + i];
+        }
+    }
+#pragma unroll
+    for (int v = 0; v < V; ++v) sh[w][32 * v + lane] = s[v];
     __syncthreads();
     if (w == 0) {
-        for (int k = 1; k < kRedWarps; ++k) s += sh[k][lane];
-        dw[i] += s;
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            for (int k = 1; k < kRedWarps; ++k) s[v] += sh[k][32 * v + lane];
+            dw[i + v] += s[v];
+        }
     }
 }
 
@@ -1041,7 +1060,10 @@ int lb_nn_conv3x3_wgrad(const void *x, const void *dy, float *dw, float *dbias, 
         if (cudaGetLastError() != cudaSuccess) return LB_ERR_CUDA;
         nchunk = p.nchunk;
     }
-    wgrad_reduce_kernel<<<(unsigned)(n / 32), 32 * kRedWarps, 0, s>>>(part, dw, n, nchunk);
+    if (n >= 65536)
+        wgrad_reduce_kernel<4><<<(unsigned)(n / 128), 32 * kRedWarps, 0, s>>>(part, dw, n, nchunk);
+    else
+        wgrad_reduce_kernel<1><<<(unsigned)(n / 32), 32 * kRedWarps, 0, s>>>(part, dw, n, nchunk);
     if (cudaGetLastError() != cudaSuccess) return LB_ERR_CUDA;
     if (dbias) {
         bias_grad_kernel<<<kBiasBlocks, 256, 0, s>>>(db, bpart, (size_t)nb * h * wd, cout);

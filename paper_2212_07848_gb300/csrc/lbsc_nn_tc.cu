@@ -1034,7 +1034,12 @@ cudaError_t launch_tcp_shape(const bf16 *x, const bf16 *w, const float *bias, bf
 // they are MN-major operands; a tap's pixel shift is a row shift of the x
 // operand's descriptor.  M = 128 rows of the operand with more channels (AC
 // real ones; the rows beyond them read other staged data or slack and land in
-// accumulator rows that are discarded), N = the other's NC channels.  A CTA
+// accumulator rows that are discarded), N = the other's NC channels.  Up to 64 of
+// them, the three dx of a tap row are one MMA of 3 NC columns: the N operand's blocks
+// of channels are given a stride of one pixel, which makes them its three shifts, and
+// the 128-row operand, whose reads bound an MMA this narrow, is read once for three
+// taps (8 x 512^2, the call: 64 -> 16 103 us against 195,
+// 16 -> 32 78 against 184).  A CTA
 // holds TP accumulators (all nine taps when 9 NC tensor-memory columns fit,
 // else the three of one tap row), sums a chunk of tiles into them, and writes
 // them once to its slice of the caller's workspace; a separate kernel adds the
@@ -1051,8 +1056,9 @@ __host__ __device__ constexpr int wg_ctas(int tp, int cin, int cout) {
     const bool ax = cin > cout;
     const int ac = ax ? cin : cout, nc = ax ? cout : cin;
     const int xr = tp == 9 ? 3 : 1;
-    const int slot = xr * ((144 * cin * 2 + 1023) / 1024 * 1024) + (128 * cout * 2 + 1023) / 1024 * 1024;
-    const int slack = (128 - ac) * (ax ? 144 : 128) * 2;
+    const int slot = xr * (((ax ? 128 : 144) * cin * 2 + 1023) / 1024 * 1024) +
+                     ((ax ? 144 : 128) * cout * 2 + 1023) / 1024 * 1024;
+    const int slack = (128 - ac) * 128 * 2;
     return tp * nc <= 256 && (110 * 1024 - slack) / slot >= 2 ? 2 : 1;
 }
 // Taps per CTA: all nine (their accumulators take 9 nc tensor-memory
@@ -1079,7 +1085,11 @@ struct WCfg {
     // with the matching 32-, 64- or 128-byte pattern)
     static constexpr int XBC = XC < 64 ? XC : 64, DBC = DC < 64 ? DC : 64;
     static constexpr int XSP = 2 * XBC, DSP = 2 * DBC;
-    static constexpr int XROW = 144, DROW = 128;        // pixel rows: x0-8 .. x0+135, x0 .. x0+127
+    // pixel rows staged: the N operand's are x0-8 .. x0+135, the other's x0 .. x0+127
+    static constexpr int XROW = AX ? 128 : 144, DROW = AX ? 144 : 128;
+    // FOLD: the three dx of a tap row in one MMA (N = 3 NC columns)
+    static constexpr bool FOLD = 3 * NC <= 256;
+    static_assert(FOLD || !AX, "shifts in the N operand");
     static constexpr int X_BYTES = XROW * XC * 2;       // one staged x row (what lands)
     static constexpr int D_BYTES = DROW * DC * 2;
     static constexpr int X_STRIDE = (X_BYTES + 1023) / 1024 * 1024;
@@ -1087,7 +1097,7 @@ struct WCfg {
     static constexpr int A_BYTES = AX ? XR * X_STRIDE : D_STRIDE;   // per slot
     static constexpr int B_BYTES = AX ? D_STRIDE : XR * X_STRIDE;
     // what the MMAs read of the A operand past its AC channels (M = 128)
-    static constexpr int SLACK = (128 - AC) * (AX ? XROW : DROW) * 2;
+    static constexpr int SLACK = (128 - AC) * 128 * 2;
     static constexpr int S0 = ((PER_SM == 2 ? 110 : 200) * 1024 - SLACK) / (A_BYTES + B_BYTES);
     static constexpr int S = S0 > 4 ? 4 : S0;           // ring slots
     static constexpr int SMEM = S * (A_BYTES + B_BYTES) + SLACK;
@@ -1113,12 +1123,13 @@ __device__ __forceinline__ uint32_t mn_desc_lo(uint32_t base, int rows) {
     return ((base & 0x3FFFFu) >> 4) | ((((uint32_t)(rows * SP) >> 4) & 0x3FFFu) << 16);
 }
 
-// tm_x / tm_xh: x as [nb*H][W][Cin], boxes of XB channels x 128 / 8 pixels;
-// tm_dy: dy as [nb*H][W][Cout], box DB channels x 128 pixels.  part: this
-// launch's partial sums [chunk][9][Cout][Cin].
+// tm_x: x as [nb*H][W][Cin], box of XB channels x 128 pixels; tm_dy: dy as
+// [nb*H][W][Cout], box DB channels x 128 pixels; tm_h: the N operand's tensor with a
+// box of 8 pixels (its halo).  part: this launch's partial sums
+// [chunk][9][Cout][Cin].
 template <int AC, int NC, bool AX>
 __global__ void __launch_bounds__(kWgtThreads, 1)
-wgrad_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_xh,
+wgrad_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_h,
                 const __grid_constant__ CUtensorMap tm_dy, float *__restrict__ part, int nb, int H,
                 int W, int Cin, int Cout, int tiles_per_chunk) {
     using C = WCfg<AC, NC, AX>;
@@ -1137,7 +1148,7 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
     };
     auto dreg = [&](int slot) { return AX ? sB + slot * C::B_BYTES : sA + slot * C::A_BYTES; };
     // both operands MN-major (bits 15 and 16)
-    constexpr uint32_t IDESC = idesc_bf16(128, NC) | (1u << 15) | (1u << 16);
+    constexpr uint32_t IDESC = idesc_bf16(128, (C::FOLD ? 3 : 1) * NC) | (1u << 15) | (1u << 16);
     const int tg = blockIdx.x % C::TG, chunk = blockIdx.x / C::TG;
     const int bands = W / 128;
     const long ntiles = (long)nb * bands * H;
@@ -1193,14 +1204,21 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
                     uint8_t *dst = xreg(slot, q);
                     for (int kc = 0; kc < C::XC / XB; ++kc) {
                         uint8_t *ch = dst + kc * C::XROW * XP;
-                        tma_load3(ch, &tm_xh, kc * XB, xl, b * H + ys, &full[slot]);
-                        tma_load3(ch + 8 * XP, &tm_x, kc * XB, x0, b * H + ys, &full[slot]);
-                        tma_load3(ch + 136 * XP, &tm_xh, kc * XB, xr, b * H + ys, &full[slot]);
+                        tma_load3(ch + (AX ? 0 : 8 * XP), &tm_x, kc * XB, x0, b * H + ys, &full[slot]);
+                        if (!AX) {
+                            tma_load3(ch, &tm_h, kc * XB, xl, b * H + ys, &full[slot]);
+                            tma_load3(ch + 136 * XP, &tm_h, kc * XB, xr, b * H + ys, &full[slot]);
+                        }
                     }
                 }
-                for (int kc = 0; kc < C::DC / DB; ++kc)
-                    tma_load3(dreg(slot) + kc * C::DROW * DP, &tm_dy, kc * DB, x0, b * H + y,
-                              &full[slot]);
+                for (int kc = 0; kc < C::DC / DB; ++kc) {
+                    uint8_t *ch = dreg(slot) + kc * C::DROW * DP;
+                    tma_load3(ch + (AX ? 8 * DP : 0), &tm_dy, kc * DB, x0, b * H + y, &full[slot]);
+                    if (AX) {
+                        tma_load3(ch, &tm_h, kc * DB, xl, b * H + y, &full[slot]);
+                        tma_load3(ch + 136 * DP, &tm_h, kc * DB, xr, b * H + y, &full[slot]);
+                    }
+                }
             }
             // every copy issued must land before the CTA exits
             for (int sq = t > S ? t - S : 0; sq < t; ++sq)
@@ -1220,27 +1238,36 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
                 ok = mbar_wait_ab(&full[slot], (uint32_t)((t / S) & 1), limit, abort);
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t d_lo = mn_desc_lo<C::DSP>(smem_u32(dreg(slot)), C::DROW);
+                // FOLD: the N operand's blocks of NC channels are one pixel row apart,
+                // so that one MMA takes the K pixels against three shifts of it
+                const uint32_t d_lo = mn_desc_lo<C::DSP>(smem_u32(dreg(slot)), AX ? 1 : C::DROW);
                 uint32_t x_lo[NQ];
 #pragma unroll
-                for (int q = 0; q < NQ; ++q) x_lo[q] = mn_desc_lo<C::XSP>(smem_u32(xreg(slot, q)), C::XROW);
+                for (int q = 0; q < NQ; ++q)
+                    x_lo[q] = mn_desc_lo<C::XSP>(smem_u32(xreg(slot, q)), C::FOLD && !AX ? 1 : C::XROW);
                 // K steps outer, taps inner: consecutive MMAs go to different
                 // accumulators, so none waits for the one before it
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    const uint32_t dd = d_lo + (uint32_t)((16 * j * C::DSP) >> 4);
+                    const uint32_t acc = (t > 0 || j > 0) ? 1u : 0u;
 #pragma unroll
-                    for (int tl = 0; tl < TP; ++tl) {
-                        // pixels 16j .. 16j+15 of the tile; x shifted by the tap
-                        // (staged row 8 is pixel x0, so the tap's row 7 + dx + p)
+                    for (int tl = 0; tl < TP; tl += C::FOLD ? 3 : 1) {
                         const int q = TP == 9 ? tl / 3 : 0, dx = tl % 3;
-                        const uint32_t xd = x_lo[q] + (uint32_t)(((7 + dx + 16 * j) * C::XSP) >> 4);
-                        if constexpr (AX)
-                            tc_mma_lo(tmem + (uint32_t)(tl * NC), xd, XHI, dd, DHI, IDESC,
-                                      (t > 0 || j > 0) ? 1u : 0u);
-                        else
-                            tc_mma_lo(tmem + (uint32_t)(tl * NC), dd, DHI, xd, XHI, IDESC,
-                                      (t > 0 || j > 0) ? 1u : 0u);
+                        if constexpr (AX) {
+                            // x pixels 16j .. 16j+15 of the tile against dy one pixel to
+                            // the right, in place and to the left (dx = 2, 1, 0): staged
+                            // row 8 is pixel x0, and accumulator tl + i belongs to dx = 2 - i
+                            tc_mma_lo(tmem + (uint32_t)(tl * NC),
+                                      x_lo[q] + (uint32_t)((16 * j * C::XSP) >> 4), XHI,
+                                      d_lo + (uint32_t)(((7 + 16 * j) * C::DSP) >> 4), DHI, IDESC, acc);
+                        } else {
+                            // dy pixels 16j .. 16j+15 of the tile against x shifted by
+                            // the tap (staged row 8 is pixel x0: row 7 + dx + p)
+                            tc_mma_lo(tmem + (uint32_t)(tl * NC),
+                                      d_lo + (uint32_t)((16 * j * C::DSP) >> 4), DHI,
+                                      x_lo[q] + (uint32_t)(((7 + dx + 16 * j) * C::XSP) >> 4), XHI,
+                                      IDESC, acc);
+                        }
                     }
                 }
                 tc_commit(&slot_free[slot]);
@@ -1276,7 +1303,7 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
             constexpr int CH = NC < 32 ? NC : 32;   // columns per tensor-memory load
 #pragma unroll 1
             for (int tl = 0; tl < TP; ++tl) {
-                const int tap = TP == 9 ? tl : tg * 3 + tl;
+                const int tap = (TP == 9 ? tl / 3 : tg) * 3 + (AX ? 2 - tl % 3 : tl % 3);
                 float *dst = part + ((size_t)chunk * 9 + tap) * Cout * Cin;
 #pragma unroll
                 for (int col = 0; col < NC; col += CH) {
@@ -1322,9 +1349,10 @@ cudaError_t launch_wgrad_t(const bf16 *x, const bf16 *dy, float *part, int nb, i
     static_assert(C::SMEM + 1024 <= 226 * 1024, "shared-memory plan too large");
     if ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(dy)) & 15)
         return cudaErrorNotSupported;
-    CUtensorMap mx, mxh, mdy;
+    CUtensorMap mx, mh, mdy;
     if (!tcp_map_span(&mx, x, cin, wd, (uint64_t)nb * h, C::XBC, 128, C::XSP) ||
-        !tcp_map_span(&mxh, x, cin, wd, (uint64_t)nb * h, C::XBC, 8, C::XSP) ||
+        !(AX ? tcp_map_span(&mh, dy, cout, wd, (uint64_t)nb * h, C::DBC, 8, C::DSP)
+             : tcp_map_span(&mh, x, cin, wd, (uint64_t)nb * h, C::XBC, 8, C::XSP)) ||
         !tcp_map_span(&mdy, dy, cout, wd, (uint64_t)nb * h, C::DBC, 128, C::DSP))
         return cudaErrorNotSupported;
     static bool attr = false;
@@ -1337,7 +1365,7 @@ cudaError_t launch_wgrad_t(const bf16 *x, const bf16 *dy, float *part, int nb, i
     const long ntiles = (long)nb * h * (wd / 128);
     const int per = (int)((ntiles + nchunk - 1) / nchunk);
     wgrad_tc_kernel<AC, NC, AX><<<C::TG * nchunk, kWgtThreads, kSmem, s>>>(
-        mx, mxh, mdy, part, nb, h, wd, cin, cout, per);
+        mx, mh, mdy, part, nb, h, wd, cin, cout, per);
     return cudaGetLastError();
 }
 

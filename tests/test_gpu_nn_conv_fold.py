@@ -62,3 +62,24 @@ def test_input_gradient(nb, h, w, cin, cout):
                            None) == 0
     assert torch.equal(out[0], out[1])
     assert L.lb_nn_status() == abi.LB_OK
+
+
+@pytest.mark.parametrize("cout", [16, 32, 64, 128])
+@pytest.mark.parametrize("cin", [16, 32, 64, 128])
+@pytest.mark.parametrize("nb,h,w", SIZES)
+def test_weight_gradient(nb, h, w, cin, cout):
+    """Whole numbers below 2^24 in every sum: equal to the FP64 sums."""
+    from paper_2212_07848_gb300 import abi
+    L = abi.load()
+    g = torch.Generator(device="cpu").manual_seed(6)
+    x, dy = (torch.randint(-3, 4, (nb, h, w, c), generator=g).bfloat16().cuda() for c in (cin, cout))
+    dw = torch.zeros((9, cout, cin), device="cuda")
+    size = L.lb_nn_wgrad_workspace(nb, h, w, cin, cout)
+    ws = torch.empty(size, dtype=torch.uint8, device="cuda")
+    assert L.lb_nn_conv3x3_wgrad(_p(x), _p(dy), _p(dw), None, nb, h, w, cin, cout, _p(ws), size,
+                                 None) == 0
+    d = dy.double().reshape(-1, cout)
+    for tap in range(9):
+        s = torch.roll(x, (1 - tap // 3, 1 - tap % 3), (1, 2)).double().reshape(-1, cin)
+        assert torch.equal(dw[tap].double(), d.t() @ s), tap
+    assert L.lb_nn_status() == abi.LB_OK
