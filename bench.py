@@ -694,7 +694,7 @@ def run_gpu(args, rank, world, local_rank):
                        "parallelism": f"replicas x{world}"},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "peak_kind": peak_kind,
-                         "kernel": "step_kernel_ov<float,4> (unit relaxation)",
+                         "kernel": "step_kernel_pair<4> (unit relaxation)",
                          "kernel_ms": k1_ms, "bytes_per_site": BYTES_PER_SITE,
                          "traffic": _step_kernel_traffic()},
             "e2e": {"value": e2e_value, "unit": "MLUPS",
