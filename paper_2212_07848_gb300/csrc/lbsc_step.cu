@@ -20,9 +20,9 @@
 // B/site, 0.95 of the measured copy rate; one column per thread in 128-column
 // strips with scalar arithmetic took 220 us, bound by issue: 391 instructions a
 // site against about 265 now, by the packed FP32 instructions, the shared
-// addresses and the 8-byte accesses) and by issue and resident warps below that.
-// 96 registers (ten 64-thread groups an SM) is the fewest without spills on the
-// unit-relaxation path: eleven and more groups measured 237-290 us, eight 217.
+// addresses and the 8-byte accesses) and by issue and resident warps below that.  96 registers (ten 64-thread groups an SM) is the fewest without
+// spills on the unit-relaxation path: eleven and more groups measured 237-290 us,
+// eight 217.
 //
 // step_kernel_pair_tile (FP32, smaller lattices): one thread per pair of sites of a
 // 32 x 8 tile, all rows at once.  A strip sweep is one long dependent program
@@ -60,32 +60,6 @@ step_kernel_pair(const KParams<float> p, const PairShape shape) {
                                               p.strip_h, p.ny);
 }
 
-// The tile kernels are launched before the grid ahead of them in the stream has ended
-// (launch_early): their CTAs come up beside its last ones and wait for its end and its
-// stores before they touch memory.  A CTA lets the next launch come up once its own
-// pulls are done (at its start instead: 1024^2 1% slower).  20 single steps of 64^2
-// 54.3 -> 51.2 us, 100 steps of 1024^2 in captured windows 1546 -> 1496 us.
-__device__ __forceinline__ void after_previous_grid() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-}
-__device__ __forceinline__ void let_next_grid_up() {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-template <typename K>
-static cudaError_t launch_early(void (*kernel)(const K), dim3 grid, int threads, cudaStream_t s,
-                                const K &k) {
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.stream = s;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, k);
-}
-
 // FP64: one thread per site of a TX x TY tile, every row at once.  The tile's ring
 // of halo pseudopotentials, H wide, is recomputed by the CTA's first threads; one
 // barrier, no row loop.
@@ -110,7 +84,6 @@ __global__ void __launch_bounds__(TX *TY) step_kernel_tile(const KParams<T> p) {
              y == 0 ? ny - 1 : y - 1, y == ny - 1 ? 0 : y + 1, g);
     };
     const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
-    after_previous_grid();
     T g[9];
     int x, y;
     pull_at(tx, ty, g, x, y);
@@ -132,7 +105,6 @@ __global__ void __launch_bounds__(TX *TY) step_kernel_tile(const KParams<T> p) {
     }
     s_psi[ty + H][tx + H] = delta_psi(sum9(g), p.psi_kind, p.rho0, p.psi_c, p.psi_b);
     __syncthreads();
-    let_next_grid_up();
     if (x0 + tx >= nx || y0 + ty >= ny) return;
     auto at = [&](int ex, int ey) { return s_psi[ty + H + ey][tx + H + ex]; };
     T sx, sy;
@@ -158,12 +130,14 @@ template <typename T, int ORDER, int TX, int TY>
 static cudaError_t launch_tile_t(const StepArgs &a, cudaStream_t s) {
     const KParams<T> k = make_params<T>(a);
     const dim3 grid((a.nx + TX - 1) / TX, (a.ny + TY - 1) / TY);
-    auto kernel = k.unit ? step_kernel_tile<T, ORDER, false, true, TX, TY>
-                         : step_kernel_tile<T, ORDER, false, false, TX, TY>;
-    if (a.drho_out)
-        kernel = k.unit ? step_kernel_tile<T, ORDER, true, true, TX, TY>
-                        : step_kernel_tile<T, ORDER, true, false, TX, TY>;
-    return launch_early(kernel, grid, TX * TY, s, k);
+    if (k.unit) {
+        if (a.drho_out) step_kernel_tile<T, ORDER, true, true, TX, TY><<<grid, TX * TY, 0, s>>>(k);
+        else step_kernel_tile<T, ORDER, false, true, TX, TY><<<grid, TX * TY, 0, s>>>(k);
+    } else {
+        if (a.drho_out) step_kernel_tile<T, ORDER, true, false, TX, TY><<<grid, TX * TY, 0, s>>>(k);
+        else step_kernel_tile<T, ORDER, false, false, TX, TY><<<grid, TX * TY, 0, s>>>(k);
+    }
+    return cudaGetLastError();
 }
 
 // The same tile in packed FP32: TX x TY sites by TX / 2 x TY threads, two neighbouring
@@ -197,7 +171,6 @@ step_kernel_pair_tile(const KParams<float> p) {
         if (i + 4 < W) s_b[j + H][i + 4] = d.y;
     };
     const int tid = threadIdx.x, tx = 2 * (tid % (TX / 2)), ty = tid / (TX / 2);
-    after_previous_grid();
     float2 g[9];
     int x, y;
     pull_at(tx, ty, g, x, y);
@@ -219,7 +192,6 @@ step_kernel_pair_tile(const KParams<float> p) {
     }
     put(tx, ty, delta_psi(sum9(g), p.psi_kind, p.rho0, p.psi_c, p.psi_b));
     __syncthreads();
-    let_next_grid_up();
     if (x0 + tx >= nx || y0 + ty >= ny) return;
     auto at = [&](int ex, int ey) {
         const float *a = s_a[ty + H + ey] + tx + 2, *b = s_b[ty + H + ey] + tx + 2;
@@ -251,12 +223,14 @@ static cudaError_t launch_pair_tile_t(const StepArgs &a, cudaStream_t s) {
     const KParams<float> k = make_params<float>(a);
     const dim3 grid((a.nx + TX - 1) / TX, (a.ny + TY - 1) / TY);
     constexpr int N = TX / 2 * TY;
-    auto kernel = k.unit ? step_kernel_pair_tile<ORDER, false, true, TX, TY>
-                         : step_kernel_pair_tile<ORDER, false, false, TX, TY>;
-    if (a.drho_out)
-        kernel = k.unit ? step_kernel_pair_tile<ORDER, true, true, TX, TY>
-                        : step_kernel_pair_tile<ORDER, true, false, TX, TY>;
-    return launch_early(kernel, grid, N, s, k);
+    if (k.unit) {
+        if (a.drho_out) step_kernel_pair_tile<ORDER, true, true, TX, TY><<<grid, N, 0, s>>>(k);
+        else step_kernel_pair_tile<ORDER, false, true, TX, TY><<<grid, N, 0, s>>>(k);
+    } else {
+        if (a.drho_out) step_kernel_pair_tile<ORDER, true, false, TX, TY><<<grid, N, 0, s>>>(k);
+        else step_kernel_pair_tile<ORDER, false, false, TX, TY><<<grid, N, 0, s>>>(k);
+    }
+    return cudaGetLastError();
 }
 
 template <int ORDER, int NT>
