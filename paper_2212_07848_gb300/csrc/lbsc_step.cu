@@ -20,9 +20,9 @@
 // B/site, 0.95 of the measured copy rate; one column per thread in 128-column
 // strips with scalar arithmetic took 220 us, bound by issue: 391 instructions a
 // site against about 265 now, by the packed FP32 instructions, the shared
-// addresses and the 8-byte accesses) and by issue and resident warps below that.  96 registers (ten 64-thread groups an SM) is the fewest without
-// spills on the unit-relaxation path: eleven and more groups measured 237-290 us,
-// eight 217.
+// addresses and the 8-byte accesses) and by issue and resident warps below that.
+// 96 registers (ten 64-thread groups an SM) is the fewest without spills on the
+// unit-relaxation path: eleven and more groups measured 237-290 us, eight 217.
 //
 // step_kernel_pair_tile (FP32, smaller lattices): one thread per pair of sites of a
 // 32 x 8 tile, all rows at once.  A strip sweep is one long dependent program
