@@ -781,8 +781,11 @@ __global__ void mse_ch_kernel(const bf16 *__restrict__ y, int C, int ch,
 // Residual MSE: prediction = base + y[.][0] (FP32 base, BF16 increment),
 // loss += mean((prediction - target)^2), dy = d loss / d y (channel 0; 0 elsewhere).
 // VEC (C a multiple of 8, dy 16-byte aligned): a pixel's channels leave as 16-byte
-// stores.  One atomic per block.  8 x 512^2, 16 channels: 47 us against
-// 174 us with 2-byte stores and an atomic per warp; bound by dy's bytes.
+// stores.  The loss is the FP32 sum of one term per warp (32 terms d^2 added by
+// halves, over n): what a term loses to the running sum's last place depends on the
+// term, so another grouping is another loss in the sixth digit (a term per block: 48
+// us for 68, and losses up to 8e-6 from these).  8 x 512^2, 16 channels: 68 us against
+// 176 us with 2-byte stores; bound by the atomics on one address (8 channels 62 us).
 template <bool VEC>
 __global__ void __launch_bounds__(256)
 mse_kernel(const bf16 *__restrict__ y, int C, const float *__restrict__ tgt,
@@ -808,14 +811,8 @@ mse_kernel(const bf16 *__restrict__ y, int C, const float *__restrict__ tgt,
             }
         }
     }
-    __shared__ float red[8];
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < 8; ++w) s += red[w];
-        atomicAdd(loss, s / (float)n);
-    }
+    if ((threadIdx.x & 31) == 0) atomicAdd(loss, s / (float)n);
 }
 
 // Mean of channel 0 of y [n][C] in two passes with a fixed summation order:
