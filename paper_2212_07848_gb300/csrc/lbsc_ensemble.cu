@@ -41,16 +41,20 @@ namespace {
 
 // Threads per group (two columns each, step_pair) and groups per SM of a layout.
 __host__ __device__ constexpr int ens_threads(bool ov) { return ov ? 128 : 64; }
-__host__ __device__ constexpr int ens_minb(bool ov, int order) {
-    return (order == 4 ? 10 : 8) * 64 / ens_threads(ov);
+// The general path keeps nine values of a row instead of three or four: at 640
+// threads an SM E4 spills 48-124 bytes a thread (96 x 128^2, tau 0.9, persistent,
+// tiles of 32 rows: 59 us a step, 45 at 512 threads with at most 20 bytes spilled).
+__host__ __device__ constexpr int ens_minb(bool ov, int order, bool unit) {
+    return (order == 4 && unit ? 10 : 8) * 64 / ens_threads(ov);
 }
 
-// UM: 1 every replica takes the unit path (all rates 1), 0 none does, 2 each
-// replica by its own rates.  One strip variant per kernel (two for UM 2): more
-// inlined variants push the strip past the register budget that the launch bounds
-// leave, and it spills.
-template <int ORDER, bool OV, int UM, bool SAMPLE>
-__global__ void __launch_bounds__(ens_threads(OV), ens_minb(OV, ORDER))
+// UNIT: every tiled replica has rates of 1 and keeps only the conserved moments of
+// the pulled rows.  One other replica and all take the general path, which is the
+// same arithmetic with gamma = 0 (see collide_tail): a kernel with both paths, each
+// replica by its own rates, spills and alternates between two bodies of code (304 x
+// 64^2 E8, every second tau 0.9: 62.5 us a step, 36.0 where all are general).
+template <int ORDER, bool OV, bool UNIT, bool SAMPLE>
+__global__ void __launch_bounds__(ens_threads(OV), ens_minb(OV, ORDER, UNIT))
 ens_step_kernel(const EnsRep *__restrict__ reps, const EnsTile *__restrict__ tiles, int ntiles,
                 EnsClock *clk, int *flag, const EnsKeys keys) {
     __shared__ KParams<float> sp;
@@ -66,19 +70,8 @@ ens_step_kernel(const EnsRep *__restrict__ reps, const EnsTile *__restrict__ til
         s_cur = cur;
     }
     __syncthreads();
-    // replicas with every relaxation rate 1 (tau = 1) take the unit path,
-    // which keeps only the conserved moments of the pulled rows
-    constexpr int NT = ens_threads(OV);
-#define ENS_STRIP(U)                                                                           \
-    step_pair<ORDER, SAMPLE, false, U, NT>(sp, keys.rk, tile.shape, tile.x0, tile.y0, tile.h,  \
-                                           tile.y1)
-    if (UM == 2) {
-        if (sp.unit) ENS_STRIP(true);
-        else ENS_STRIP(false);
-    } else {
-        ENS_STRIP(UM == 1);
-    }
-#undef ENS_STRIP
+    step_pair<ORDER, SAMPLE, false, UNIT, ens_threads(OV)>(sp, keys.rk, tile.shape, tile.x0,
+                                                           tile.y0, tile.h, tile.y1);
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
@@ -155,10 +148,10 @@ __device__ int wait_tiles(const uint32_t *tdone, const int *__restrict__ nbr, in
     }
 }
 
-// UM as in ens_step_kernel.  The persistent launch never samples; a sampling step
+// UNIT as in ens_step_kernel.  The persistent launch never samples; a sampling step
 // runs through the per-step kernel.
-template <int ORDER, bool OV, int UM>
-__global__ void __launch_bounds__(ens_threads(OV), ens_minb(OV, ORDER))
+template <int ORDER, bool OV, bool UNIT>
+__global__ void __launch_bounds__(ens_threads(OV), ens_minb(OV, ORDER, UNIT))
 ens_persist_kernel(const EnsRep *__restrict__ reps, const EnsTile *__restrict__ tiles,
                    int ntiles, const int *__restrict__ nbr_off, const int *__restrict__ nbr,
                    uint32_t *tdone, EnsCtl *ctl, EnsClock *clk, int *flag, const EnsKeys keys,
@@ -214,17 +207,8 @@ ens_persist_kernel(const EnsRep *__restrict__ reps, const EnsTile *__restrict__ 
         }
         __syncthreads();
         if (!s_go) break;
-        constexpr int NT = ens_threads(OV);
-#define ENS_STRIP(U)                                                                            \
-    step_pair<ORDER, false, true, U, NT>(sp, keys.rk, s_tile.shape, s_tile.x0, s_tile.y0,       \
-                                         s_tile.h, s_tile.y1)
-        if (UM == 2) {
-            if (sp.unit) ENS_STRIP(true);
-            else ENS_STRIP(false);
-        } else {
-            ENS_STRIP(UM == 1);
-        }
-#undef ENS_STRIP
+        step_pair<ORDER, false, true, UNIT, ens_threads(OV)>(
+            sp, keys.rk, s_tile.shape, s_tile.x0, s_tile.y0, s_tile.h, s_tile.y1);
         if (threadIdx.x == 0) s_k[it ^ 1] = knext;
         // read before the barrier: thread 0 overwrites s_ti after it
         const int ti = s_ti;
@@ -341,7 +325,7 @@ struct lb_ens {
     int persist_grid = 0;                      // co-resident CTAs of the persistent kernel
     int kernel_mode = LB_KERNEL_AUTO;          // LB_KERNEL_PLAIN or _OVERLAP (strip layout)
     bool ov = false;                           // the layout in use
-    int umode = 2;                             // unit path: 1 every replica, 0 none, 2 mixed
+    bool unit = false;                         // every tiled replica has rates of 1
     int resident_mode = LB_ENS_RESIDENT_AUTO;  // which replicas live in shared memory
     std::vector<ResClass> rclasses;            // resident replicas, one launch per shape
     std::vector<char> is_res;                  // replica r is resident
@@ -476,6 +460,8 @@ int setup_resident(lb_ens *e) {
     return LB_OK;
 }
 
+cudaError_t persist_occupancy(lb_ens *e);
+
 int build_tiles(lb_ens *e) {
     std::vector<EnsTile> tiles;
     std::vector<int> order(e->nrep);
@@ -488,6 +474,9 @@ int build_tiles(lb_ens *e) {
     // (periodic); the tiles holding those cells are its dependencies in the
     // persistent launch (CSR: nbr_off, nbr).
     const int H = e->stencil == 4 ? 1 : 2;
+    e->unit = true;
+    for (int r : order) e->unit = e->unit && (e->is_res[r] || e->h_reps[r].unit);
+    ENS_CHECK(persist_occupancy(e));
     std::vector<int> nbr_off(1, 0), nbr;
     for (int r : order) {
         if (e->is_res[r]) continue;   // advanced by the resident kernel
@@ -545,27 +534,26 @@ int build_tiles(lb_ens *e) {
     return LB_OK;
 }
 
-template <int ORDER, bool OV, int UM>
+template <int ORDER, bool OV, bool UNIT>
 cudaError_t launch_persist_t(lb_ens *e, int nsteps) {
     void *args[] = {&e->d_reps,  &e->d_tiles, &e->ntiles, &e->d_nbr_off, &e->d_nbr,
                     &e->d_tdone, &e->d_ctl,   &e->d_clk,  &e->d_flag,    &e->keys,
                     &nsteps};
     const int grid = std::min(e->persist_grid, e->ntiles);
-    return cudaLaunchCooperativeKernel((const void *)ens_persist_kernel<ORDER, OV, UM>,
+    return cudaLaunchCooperativeKernel((const void *)ens_persist_kernel<ORDER, OV, UNIT>,
                                        dim3(grid), dim3(ens_threads(OV)), args, 0,
                                        e->stream);
 }
 
-// The persistent kernel of the ensemble's stencil, layout and unit mode.
+// The persistent kernel of the ensemble's stencil, layout and path.
 template <int ORDER, bool OV>
-const void *persist_fn_ov(int um) {
-    return um == 1   ? (const void *)ens_persist_kernel<ORDER, OV, 1>
-           : um == 0 ? (const void *)ens_persist_kernel<ORDER, OV, 0>
-                     : (const void *)ens_persist_kernel<ORDER, OV, 2>;
+const void *persist_fn_ov(bool unit) {
+    return unit ? (const void *)ens_persist_kernel<ORDER, OV, true>
+                : (const void *)ens_persist_kernel<ORDER, OV, false>;
 }
 template <int ORDER>
 const void *persist_fn_o(const lb_ens *e) {
-    return e->ov ? persist_fn_ov<ORDER, true>(e->umode) : persist_fn_ov<ORDER, false>(e->umode);
+    return e->ov ? persist_fn_ov<ORDER, true>(e->unit) : persist_fn_ov<ORDER, false>(e->unit);
 }
 const void *persist_fn(const lb_ens *e) {
     return e->stencil == 4   ? persist_fn_o<4>(e)
@@ -575,9 +563,8 @@ const void *persist_fn(const lb_ens *e) {
 
 template <int ORDER, bool OV>
 cudaError_t launch_persist_ov(lb_ens *e, int nsteps) {
-    return e->umode == 1   ? launch_persist_t<ORDER, OV, 1>(e, nsteps)
-           : e->umode == 0 ? launch_persist_t<ORDER, OV, 0>(e, nsteps)
-                           : launch_persist_t<ORDER, OV, 2>(e, nsteps);
+    return e->unit ? launch_persist_t<ORDER, OV, true>(e, nsteps)
+                   : launch_persist_t<ORDER, OV, false>(e, nsteps);
 }
 template <int ORDER>
 cudaError_t launch_persist_o(lb_ens *e, int nsteps) {
@@ -614,25 +601,23 @@ cudaError_t launch_ens_persistent(lb_ens *e, int nsteps, bool sample_last) {
     return launch_ens_step(e, true);
 }
 
-template <int ORDER, bool OV, int UM>
+template <int ORDER, bool OV, bool UNIT>
 void launch_ens_step_t(lb_ens *e, bool sample) {
     if (sample)
-        ens_step_kernel<ORDER, OV, UM, true><<<e->ntiles, ens_threads(OV), 0, e->stream>>>(
+        ens_step_kernel<ORDER, OV, UNIT, true><<<e->ntiles, ens_threads(OV), 0, e->stream>>>(
             e->d_reps, e->d_tiles, e->ntiles, e->d_clk, e->d_flag, e->keys);
     else
-        ens_step_kernel<ORDER, OV, UM, false><<<e->ntiles, ens_threads(OV), 0, e->stream>>>(
+        ens_step_kernel<ORDER, OV, UNIT, false><<<e->ntiles, ens_threads(OV), 0, e->stream>>>(
             e->d_reps, e->d_tiles, e->ntiles, e->d_clk, e->d_flag, e->keys);
 }
 template <int ORDER>
 void launch_ens_step_o(lb_ens *e, bool sample) {
     if (e->ov) {
-        if (e->umode == 1) launch_ens_step_t<ORDER, true, 1>(e, sample);
-        else if (e->umode == 0) launch_ens_step_t<ORDER, true, 0>(e, sample);
-        else launch_ens_step_t<ORDER, true, 2>(e, sample);
+        if (e->unit) launch_ens_step_t<ORDER, true, true>(e, sample);
+        else launch_ens_step_t<ORDER, true, false>(e, sample);
     } else {
-        if (e->umode == 1) launch_ens_step_t<ORDER, false, 1>(e, sample);
-        else if (e->umode == 0) launch_ens_step_t<ORDER, false, 0>(e, sample);
-        else launch_ens_step_t<ORDER, false, 2>(e, sample);
+        if (e->unit) launch_ens_step_t<ORDER, false, true>(e, sample);
+        else launch_ens_step_t<ORDER, false, false>(e, sample);
     }
 }
 
@@ -805,13 +790,6 @@ int lb_ens_create(lb_ens **out, const lb_replica *reps, int nrep, int psi_kind, 
         const EnsCtl c0 = {0u, 0, (unsigned long long)kEnsWaitNs, 0u};
         err = cudaMemcpy(e->d_ctl, &c0, sizeof(EnsCtl), cudaMemcpyHostToDevice);
     }
-    {
-        // a replica takes the unit path when its rates are 1 (fold_rates)
-        int nunit = 0;
-        for (int r = 0; r < nrep; ++r) nunit += 1.0 - 1.0 / reps[r].tau == 0.0;
-        e->umode = nunit == nrep ? 1 : nunit == 0 ? 0 : 2;
-    }
-    if (err == cudaSuccess) err = persist_occupancy(e);
     if (err != cudaSuccess) {
         free_ens(e);
         delete e;
@@ -970,7 +948,6 @@ int lb_ens_set_kernel(lb_ens *e, int mode) {
     // {64..512}^2, persistent: 256 against 250 us a step, both 336 us with one column
     // per thread) but is slower for 32^2.
     e->ov = mode == LB_KERNEL_OVERLAP;
-    ENS_CHECK(persist_occupancy(e));
     return build_tiles(e);
 }
 

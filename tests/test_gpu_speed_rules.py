@@ -1,0 +1,46 @@
+"""Choices of a path whose wrong side costs 1.5 times and more, by the ratio of two calls
+timed in turn on the same device (medians; the limits lie between the two sides)."""
+import time
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+LN2 = float(np.log(2.0))
+
+
+def _times(objs, calls, rounds=9):
+    """Median seconds of each call, the calls taken in turn."""
+    got = [[] for _ in calls]
+    for k in range(rounds + 2):
+        for i, (o, call) in enumerate(zip(objs, calls)):
+            o.sync()
+            t = time.perf_counter()
+            call()
+            o.sync()
+            if k >= 2:
+                got[i].append(time.perf_counter() - t)
+    return [sorted(g)[len(g) // 2] for g in got]
+
+
+def _ensemble(n, nrep, taus, stencil, launch, resident):
+    from paper_2212_07848_gb300.ensemble import Ensemble
+    e = Ensemble([(n, n, -3.6 - 0.0005 * r, taus[r % len(taus)], 1e-6, LN2) for r in range(nrep)],
+                 stencil=stencil, seed=3)
+    e.set_resident(resident)
+    e.set_launch(launch)
+    e.init(1e-3)
+    return e
+
+
+@pytest.mark.parametrize("stencil", [4, 8])
+@pytest.mark.parametrize("launch", ["LB_ENS_PER_STEP", "LB_ENS_PERSISTENT"])
+def test_ensembles_of_mixed_rates(launch, stencil):
+    """Every second replica at unit rates is no slower than none of them."""
+    from paper_2212_07848_gb300 import abi
+    es = [_ensemble(64, 304, taus, stencil, getattr(abi, launch), abi.LB_ENS_RESIDENT_OFF)
+          for taus in ([0.9], [1.0, 0.9])]
+    general, mixed = _times(es, [lambda e=e: e.step(64) for e in es])
+    for e in es:
+        e.close()
+    assert mixed < 1.15 * general
