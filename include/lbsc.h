@@ -306,7 +306,9 @@ void lb_ens_destroy(lb_ens *e);
 int lb_ens_init(lb_ens *e, double init_amp);
 /* Per-replica S(k) schedule, as lb_sk_config (all sizes powers of two). */
 int lb_ens_sk_config(lb_ens *e, int sample_every, long long start_step);
-/* Rows swept per CTA for every replica (tile shape). */
+/* Rows of a band of a CTA's strip, for every replica (tile shape; the default is
+ * chosen from the ensemble).  An upper bound where the tiles would not fill the
+ * GPU.  Does not change results. */
 int lb_ens_set_strip_height(lb_ens *e, int rows);
 /* Time candidate strip heights on a snapshot of the state (restored after),
  * keep the fastest, and cache it in cache_path ("key strip" lines; may be

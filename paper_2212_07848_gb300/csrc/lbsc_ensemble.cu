@@ -313,7 +313,7 @@ struct lb_ens {
     long long t = 0;
     int cur = 0;
     bool inited = false;
-    int strip_h = 32;
+    int strip_h = 0;                    // rows of a band asked for, or 0 (tile_height)
     int sk_every = 0;
     long long sk_start = 0, sk_count = 0;
     cudaGraphExec_t graph_plain = nullptr;     // kGraphSteps steps, no sampling
@@ -462,6 +462,46 @@ int setup_resident(lb_ens *e) {
 
 cudaError_t persist_occupancy(lb_ens *e);
 
+// Rows of a replica's bands where `rows` are asked for.
+int band_rows(int ny, const PairShape &shape, int rows) {
+    return std::min(rows, (ny + shape.bands - 1) / shape.bands);
+}
+// Tiles of the replicas that are not resident.
+long count_tiles(const lb_ens *e, int rows) {
+    long n = 0;
+    for (int r = 0; r < e->nrep; ++r) {
+        if (e->is_res[r]) continue;
+        const PairShape shape = pair_shape(e->reps[r].nx, ens_threads(e->ov));
+        const int h = band_rows(e->reps[r].ny, shape, rows) * shape.bands;
+        n += (long)((e->reps[r].ny + h - 1) / h) * shape.strips;
+    }
+    return n;
+}
+
+// Rows of a band when none is set: the fewest waves of resident groups that bands of
+// at most 32 rows need, then the lowest bands that fit them.  A group's rows are one
+// long dependent program (about 1 us each), so an ensemble that does not fill the SMs
+// gains from more and lower bands, and a height that is set is only an upper bound
+// there; a large one keeps 32.  us a step, 32 rows -> this, E4 at unit rates: 8 x 128^2
+// 30.3 -> 8.0 (4 rows), 16 x 256^2 36.9 -> 19.6 (6), 96 x 128^2 39.4 -> 26.6 (12), 2 x
+// 2048^2 122 -> 112 (24); 256 of {64..512}^2 269 (32; 24 rows 281, 48 rows 289).  A
+// persistent launch overlaps the steps: within a wave it gains from half as many tiles
+// again (96 x 128^2 25.5 -> 21.9, 16 x 256^2 18.6 -> 16.9), beyond one it does not (256
+// of {64..512}^2 at tau 0.9 307 -> 315).
+constexpr int kMaxHeight = 32;
+int tile_height(const lb_ens *e) {
+    int nsm = 152;
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, e->dev);
+    const long slots = (long)nsm * ens_minb(e->ov, e->stencil, e->unit);
+    if (e->strip_h > 0 && count_tiles(e, e->strip_h) >= slots) return e->strip_h;
+    const int most = e->strip_h > 0 ? std::min(e->strip_h, kMaxHeight) : kMaxHeight;
+    const long waves = (count_tiles(e, kMaxHeight) + slots - 1) / slots;
+    const bool more = waves == 1 && e->launch_mode == LB_ENS_PERSISTENT;
+    for (int h : {4, 6, 8, 12, 16, 24})
+        if (h < most && count_tiles(e, h) <= (more ? slots + slots / 2 : waves * slots)) return h;
+    return most;
+}
+
 int build_tiles(lb_ens *e) {
     std::vector<EnsTile> tiles;
     std::vector<int> order(e->nrep);
@@ -477,12 +517,13 @@ int build_tiles(lb_ens *e) {
     e->unit = true;
     for (int r : order) e->unit = e->unit && (e->is_res[r] || e->h_reps[r].unit);
     ENS_CHECK(persist_occupancy(e));
+    const int rows = tile_height(e);
     std::vector<int> nbr_off(1, 0), nbr;
     for (int r : order) {
         if (e->is_res[r]) continue;   // advanced by the resident kernel
         const int nx = e->reps[r].nx, ny = e->reps[r].ny;
         const PairShape shape = pair_shape(nx, ens_threads(e->ov));
-        const int hb = std::min(e->strip_h, (ny + shape.bands - 1) / shape.bands);
+        const int hb = band_rows(ny, shape, rows);
         const int h = hb * shape.bands, cols = shape.cols;
         const int nry = (ny + h - 1) / h, ncx = shape.strips;
         const int base = (int)tiles.size();
@@ -931,8 +972,7 @@ int lb_ens_set_launch(lb_ens *e, int mode) {
         if (!coop || e->persist_grid < 1) return LB_ERR_UNSUPPORTED;
     }
     e->launch_mode = mode;
-    drop_graphs(e);
-    return LB_OK;
+    return build_tiles(e);
 }
 
 int lb_ens_get_launch(const lb_ens *e) { return e ? e->launch_mode : LB_ERR_ARG; }
@@ -1118,7 +1158,7 @@ int lb_ens_autotune(lb_ens *e, int trial_steps, const char *cache_path, int *cho
     if (!e->inited) return LB_ERR_STATE;
     ENS_CHECK(cudaSetDevice(e->dev));
     if (e->ntiles == 0) {   // every replica resident: there is no tile shape to tune
-        if (chosen) *chosen = e->strip_h;
+        if (chosen) *chosen = e->strip_h > 0 ? e->strip_h : kMaxHeight;
         return LB_OK;
     }
     cudaDeviceProp prop;

@@ -44,3 +44,19 @@ def test_ensembles_of_mixed_rates(launch, stencil):
     for e in es:
         e.close()
     assert mixed < 1.15 * general
+
+
+@pytest.mark.parametrize("n,nrep", [(128, 8), (256, 16), (1024, 1)])
+@pytest.mark.parametrize("launch", ["LB_ENS_PER_STEP", "LB_ENS_PERSISTENT"])
+def test_default_bands_of_small_ensembles(launch, n, nrep):
+    """The default height, and a height that is set, on ensembles that tall bands leave
+    on a part of the SMs, against bands of 6 rows."""
+    from paper_2212_07848_gb300 import abi
+    es = [_ensemble(n, nrep, [1.0], 4, getattr(abi, launch), abi.LB_ENS_RESIDENT_OFF)
+          for _ in range(3)]
+    es[0].set_strip_height(6)
+    es[2].set_strip_height(32)
+    low, default, tall = _times(es, [lambda e=e: e.step(64) for e in es])
+    for e in es:
+        e.close()
+    assert default < 1.4 * low and tall < 1.4 * low
