@@ -63,14 +63,17 @@ step_kernel_pair(const KParams<float> p, const PairShape shape) {
 // FP64: one thread per site of a TX x TY tile, every row at once.  The tile's ring
 // of halo pseudopotentials, H wide, is recomputed by the CTA's first threads; one
 // barrier, no row loop.
-template <typename T, int ORDER, bool SAMPLE, bool UNIT, int TX, int TY>
-__global__ void __launch_bounds__(TX *TY) step_kernel_tile(const KParams<T> p) {
+// TALL: one of several launches over a lattice of more rows of tiles than a grid's
+// second dimension holds; its first row is row0.
+constexpr int kGridRows = 65535;
+template <typename T, int ORDER, bool SAMPLE, bool UNIT, int TX, int TY, bool TALL>
+__global__ void __launch_bounds__(TX *TY) step_kernel_tile(const KParams<T> p, const int row0) {
     constexpr int H = Stencil<ORDER>::H, W = TX + 2 * H, NT = TX * TY;
     constexpr int kRing = W * (TY + 2 * H) - NT;   // rows above and below, then the sides
     __shared__ T s_psi[TY + 2 * H][W];
     const int nx = p.nx, ny = p.ny;
     const size_t plane = (size_t)nx * ny;
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
+    const int x0 = blockIdx.x * TX, y0 = (TALL ? row0 : 0) + blockIdx.y * TY;
     // populations of the site (x0 + i, y0 + j), -H <= i < TX + H, periodic (a tile
     // may reach past the lattice's edge by more than its size)
     auto pull_at = [&](int i, int j, T g[9], int &x, int &y) {
@@ -126,17 +129,21 @@ __global__ void __launch_bounds__(TX *TY) step_kernel_tile(const KParams<T> p) {
     if (!isfinite(f[1] + f[5])) atomicOr(p.flag, LB_STEP_NONFINITE);
 }
 
-template <typename T, int ORDER, int TX, int TY>
-static cudaError_t launch_tile_t(const StepArgs &a, cudaStream_t s) {
+template <typename T, int ORDER, int TX, int TY, bool TALL = false>
+static cudaError_t launch_tile_t(const StepArgs &a, cudaStream_t s, int row0 = 0) {
     const KParams<T> k = make_params<T>(a);
-    const dim3 grid((a.nx + TX - 1) / TX, (a.ny + TY - 1) / TY);
+    const int rows = (a.ny - row0 + TY - 1) / TY;
+    const dim3 grid((a.nx + TX - 1) / TX, rows < kGridRows ? rows : kGridRows);
+#define TILE(SAMPLE, UNIT)                                                                   \
+    step_kernel_tile<T, ORDER, SAMPLE, UNIT, TX, TY, TALL><<<grid, TX * TY, 0, s>>>(k, row0)
     if (k.unit) {
-        if (a.drho_out) step_kernel_tile<T, ORDER, true, true, TX, TY><<<grid, TX * TY, 0, s>>>(k);
-        else step_kernel_tile<T, ORDER, false, true, TX, TY><<<grid, TX * TY, 0, s>>>(k);
+        if (a.drho_out) TILE(true, true);
+        else TILE(false, true);
     } else {
-        if (a.drho_out) step_kernel_tile<T, ORDER, true, false, TX, TY><<<grid, TX * TY, 0, s>>>(k);
-        else step_kernel_tile<T, ORDER, false, false, TX, TY><<<grid, TX * TY, 0, s>>>(k);
+        if (a.drho_out) TILE(true, false);
+        else TILE(false, false);
     }
+#undef TILE
     return cudaGetLastError();
 }
 
@@ -256,9 +263,16 @@ static cudaError_t launch_f32(const StepArgs &a, cudaStream_t s) {
 }
 
 // Small FP64 lattices take the smaller tile, which spreads them over more SMs
-// (128^2: 16 against 27 us; 1024^2: 1% slower).
+// (128^2: 16 against 27 us; 1024^2: 1% slower).  A lattice of more than 524280 rows
+// takes a launch for each kGridRows rows of tiles.
 template <int ORDER>
 static cudaError_t launch_f64(const StepArgs &a, cudaStream_t s) {
+    if (a.ny > 8 * kGridRows) {
+        cudaError_t e = cudaSuccess;
+        for (int r = 0; r < a.ny && e == cudaSuccess; r += 8 * kGridRows)
+            e = launch_tile_t<double, ORDER, 16, 8, true>(a, s, r);
+        return e;
+    }
     return (size_t)a.nx * a.ny < (1u << 17) ? launch_tile_t<double, ORDER, 16, 8>(a, s)
                                             : launch_tile_t<double, ORDER, 32, 8>(a, s);
 }
@@ -267,9 +281,10 @@ static cudaError_t launch_f64(const StepArgs &a, cudaStream_t s) {
 // strips have caught up.  us per step, tiles / strips: unit rates E4 1024^2 14.4 /
 // 15.4, 1500 x 1000 22.0 / 22.5, 2048^2 59.9 / 52.8; general rates E4 708 x 452 6.1 /
 // 8.0, 2048^2 62 / 67, 4096^2 238 / 234; E8 general 512^2 5.9 / 9.1, 2048^2 66 / 74,
-// 4096^2 255 / 234.
+// 4096^2 255 / 234.  Never for more rows of tiles than a grid has.
 bool tile_is_faster(int nx, int ny, bool unit) {
-    return (size_t)nx * ny <= (unit ? (size_t)3 << 19 : (size_t)1 << 23);
+    return ny <= 8 * kGridRows &&
+           (size_t)nx * ny <= (unit ? (size_t)3 << 19 : (size_t)1 << 23);
 }
 
 // Rows per band of a strip: the fewest waves of resident groups whose bands are at
