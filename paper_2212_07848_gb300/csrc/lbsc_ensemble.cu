@@ -409,6 +409,32 @@ bool resident_shape(const lb_ens *e, int nx, int ny, bool unit, int max_c, ResCl
     return false;
 }
 
+// A shape with replicas of both paths: one launch of the general path for all (the
+// same bits, see ens_step_kernel) where that takes less time than a launch for each,
+// the general path's waves of resident CTAs costing a fourth more.  152 x 64^2, every
+// second tau 0.9: 17.6 us a step in two launches of half a wave, 10.4 in one; 304
+// replicas: 17.9 in two full waves, 20.2 in one launch.
+void merge_classes(lb_ens *e, std::vector<ResClass> &cls) {
+    int nsm = 152;
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, e->dev);
+    auto waves = [&](const ResClass &c, size_t nrep) {
+        const int m = resident_max_clusters(e->stencil, c.C, c.nx, c.ny / c.C, c.unit, c.smem);
+        const size_t slots = (size_t)std::max(1, c.C == 1 ? m * nsm : m);
+        return (nrep + slots - 1) / slots;
+    };
+    for (size_t u = 0; u < cls.size(); ++u)
+        for (size_t g = 0; cls[u].unit && g < cls.size(); ++g) {
+            if (cls[g].unit || cls[g].nx != cls[u].nx || cls[g].ny != cls[u].ny) continue;
+            const size_t nu = cls[u].reps.size(), ng = cls[g].reps.size();
+            if (5 * waves(cls[g], nu + ng) <= 4 * waves(cls[u], nu) + 5 * waves(cls[g], ng)) {
+                cls[g].reps.insert(cls[g].reps.end(), cls[u].reps.begin(), cls[u].reps.end());
+                cls.erase(cls.begin() + u);
+                --u;
+            }
+            break;
+        }
+}
+
 // Which replicas live in shared memory (resident_mode): none; every one
 // whose shape allows it; or, AUTO, all of them when each fits one CTA.
 // AUTO leaves out the clusters (128^2 over four CTAs measured 64 against 83
@@ -449,6 +475,7 @@ int setup_resident(lb_ens *e) {
         cls[k].reps.push_back(r);
         ++n;
     }
+    merge_classes(e, cls);
     for (auto &c : cls) {
         ENS_CHECK(cudaMalloc(&c.d_list, c.reps.size() * sizeof(int)));
         ENS_CHECK(cudaMemcpy(c.d_list, c.reps.data(), c.reps.size() * sizeof(int),

@@ -60,3 +60,29 @@ def test_default_bands_of_small_ensembles(launch, n, nrep):
     for e in es:
         e.close()
     assert default < 1.4 * low and tall < 1.4 * low
+
+
+def test_resident_ensembles_of_mixed_rates():
+    """Replicas of both paths that fill the SMs once: not two half-empty launches."""
+    from paper_2212_07848_gb300 import abi
+    es = [_ensemble(64, 152, taus, 4, abi.LB_ENS_PER_STEP, abi.LB_ENS_RESIDENT_ON)
+          for taus in ([0.9], [1.0, 0.9])]
+    assert all(e.num_resident == 152 for e in es)
+    general, mixed = _times(es, [lambda e=e: e.step(64) for e in es])
+    for e in es:
+        e.close()
+    assert mixed < 1.25 * general
+
+
+@pytest.mark.parametrize("nrep,taus", [(5, [1.0, 0.9]), (6, [0.9, 0.9, 1.0])])
+def test_merged_residents_keep_their_bits(nrep, taus):
+    from paper_2212_07848_gb300 import abi
+    out = []
+    for mode in (abi.LB_ENS_RESIDENT_ON, abi.LB_ENS_RESIDENT_OFF):
+        e = _ensemble(32, nrep, taus, 8, abi.LB_ENS_PER_STEP, mode)
+        e.sk_config(4, 4)
+        e.step(13)
+        e.sync()
+        out.append([e.populations(r) for r in range(nrep)])
+        e.close()
+    assert all(np.array_equal(a, b) for a, b in zip(*out))
