@@ -88,6 +88,7 @@ struct ResLaunch {
     int nx, ny;             // the shape (nx in {32, 64, 128})
     int C;                  // CTAs per replica (cluster size: 1, 2, 4 or 8)
     bool unit;              // every replica of the list takes the unit path
+    bool many;              // more CTAs than SMs
     int stencil;            // 4, 6, 8
     EnsClock *clk;
     int *flag;
@@ -101,7 +102,8 @@ size_t resident_smem(int nx, int rows, int stencil);
 // Opt the kernels of (stencil, C) in to `smem` bytes of dynamic shared memory.
 cudaError_t resident_prepare(int stencil, int C, size_t smem);
 // Clusters of C CTAs (CTAs per SM when C = 1) that can be resident at once.
-int resident_max_clusters(int stencil, int C, int nx, int rows, bool unit, size_t smem);
+int resident_max_clusters(int stencil, int C, int nx, int rows, bool unit, bool many,
+                          size_t smem);
 cudaError_t launch_ens_resident(const ResLaunch &a, cudaStream_t s);
 
 }  // namespace lbsc

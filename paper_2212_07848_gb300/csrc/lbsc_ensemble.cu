@@ -395,7 +395,7 @@ bool resident_shape(const lb_ens *e, int nx, int ny, bool unit, int max_c, ResCl
             cudaGetLastError();
             return false;
         }
-        if (resident_max_clusters(e->stencil, c, nx, rows, unit, sm) < 1) {
+        if (resident_max_clusters(e->stencil, c, nx, rows, unit, false, sm) < 1) {
             cudaGetLastError();
             continue;
         }
@@ -409,16 +409,22 @@ bool resident_shape(const lb_ens *e, int nx, int ny, bool unit, int max_c, ResCl
     return false;
 }
 
+int sm_count(const lb_ens *e) {
+    int n = 152;
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, e->dev);
+    return n;
+}
+
 // A shape with replicas of both paths: one launch of the general path for all (the
 // same bits, see ens_step_kernel) where that takes less time than a launch for each,
 // the general path's waves of resident CTAs costing a fourth more.  152 x 64^2, every
 // second tau 0.9: 17.6 us a step in two launches of half a wave, 10.4 in one; 304
 // replicas: 17.9 in two full waves, 20.2 in one launch.
 void merge_classes(lb_ens *e, std::vector<ResClass> &cls) {
-    int nsm = 152;
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, e->dev);
+    const int nsm = sm_count(e);
     auto waves = [&](const ResClass &c, size_t nrep) {
-        const int m = resident_max_clusters(e->stencil, c.C, c.nx, c.ny / c.C, c.unit, c.smem);
+        const int m = resident_max_clusters(e->stencil, c.C, c.nx, c.ny / c.C, c.unit,
+                                            nrep * c.C > (size_t)nsm, c.smem);
         const size_t slots = (size_t)std::max(1, c.C == 1 ? m * nsm : m);
         return (nrep + slots - 1) / slots;
     };
@@ -517,9 +523,7 @@ long count_tiles(const lb_ens *e, int rows) {
 // of {64..512}^2 at tau 0.9 307 -> 315).
 constexpr int kMaxHeight = 32;
 int tile_height(const lb_ens *e) {
-    int nsm = 152;
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, e->dev);
-    const long slots = (long)nsm * ens_minb(e->ov, e->stencil, e->unit);
+    const long slots = (long)sm_count(e) * ens_minb(e->ov, e->stencil, e->unit);
     if (e->strip_h > 0 && count_tiles(e, e->strip_h) >= slots) return e->strip_h;
     const int most = e->strip_h > 0 ? std::min(e->strip_h, kMaxHeight) : kMaxHeight;
     const long waves = (count_tiles(e, kMaxHeight) + slots - 1) / slots;
@@ -726,6 +730,7 @@ cudaError_t launch_window(lb_ens *e, int steps, bool sample_last) {
         a.ny = c.ny;
         a.C = c.C;
         a.unit = c.unit;
+        a.many = (long)a.nres * a.C > sm_count(e);
         a.stencil = e->stencil;
         a.clk = e->d_clk;
         a.flag = e->d_flag;

@@ -243,9 +243,12 @@ const void *res_fn(int stencil, int C, bool unit) {
                           : res_fn_o<8>(C, unit);
 }
 
-// Threads of a CTA of `rows` rows: a pair of sites each, as far as they go.
-int res_block(int nx, int rows, bool unit) {
-    const int pairs = rows * nx / 2;
+// Threads of a CTA of `rows` rows: a pair of sites each, as far as they go.  On the
+// general path (128 registers) one CTA of 32^2 then fills an SM, so with more CTAs
+// than SMs (`many`) a thread takes two pairs and two CTAs overlap: 4096 x 32^2, tau
+// 0.9, 54.8 us a step against 73.3 (four pairs 58.8); 152 replicas 4.3 against 4.4.
+int res_block(int nx, int rows, bool unit, bool many) {
+    const int pairs = rows * nx / (many && !unit ? 4 : 2);
     return pairs < res_threads(unit) ? (pairs + 31) / 32 * 32 : res_threads(unit);
 }
 
@@ -269,10 +272,11 @@ cudaError_t resident_prepare(int stencil, int C, size_t smem) {
     return cudaSuccess;
 }
 
-int resident_max_clusters(int stencil, int C, int nx, int rows, bool unit, size_t smem) {
+int resident_max_clusters(int stencil, int C, int nx, int rows, bool unit, bool many,
+                          size_t smem) {
     const void *fn = res_fn(stencil, C, unit);
     if (!fn) return 0;
-    const int threads = res_block(nx, rows, unit);
+    const int threads = res_block(nx, rows, unit, many);
     if (C == 1) {
         int n = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, threads, smem) != cudaSuccess)
@@ -302,7 +306,7 @@ cudaError_t launch_ens_resident(const ResLaunch &a, cudaStream_t s) {
     const size_t smem = resident_smem(a.nx, rows, a.stencil);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(a.nres * a.C);
-    cfg.blockDim = dim3(res_block(a.nx, rows, a.unit));
+    cfg.blockDim = dim3(res_block(a.nx, rows, a.unit, a.many));
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr;

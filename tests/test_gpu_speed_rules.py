@@ -25,7 +25,7 @@ def _times(objs, calls, rounds=9):
 
 def _ensemble(n, nrep, taus, stencil, launch, resident):
     from paper_2212_07848_gb300.ensemble import Ensemble
-    e = Ensemble([(n, n, -3.6 - 0.0005 * r, taus[r % len(taus)], 1e-6, LN2) for r in range(nrep)],
+    e = Ensemble([(n, n, -3.6 - 0.0002 * r, taus[r % len(taus)], 1e-6, LN2) for r in range(nrep)],
                  stencil=stencil, seed=3)
     e.set_resident(resident)
     e.set_launch(launch)
@@ -86,3 +86,15 @@ def test_merged_residents_keep_their_bits(nrep, taus):
         out.append([e.populations(r) for r in range(nrep)])
         e.close()
     assert all(np.array_equal(a, b) for a, b in zip(*out))
+
+
+def test_many_small_residents_at_general_rates():
+    """32^2 replicas of the general path, two CTAs an SM: less than 1.4 times the unit
+    path's time (one CTA an SM: 1.6)."""
+    from paper_2212_07848_gb300 import abi
+    es = [_ensemble(32, 2000, [tau], 4, abi.LB_ENS_PER_STEP, abi.LB_ENS_RESIDENT_ON)
+          for tau in (1.0, 0.9)]
+    unit, general = _times(es, [lambda e=e: e.step(64) for e in es])
+    for e in es:
+        e.close()
+    assert general < 1.4 * unit
