@@ -71,7 +71,8 @@ extern "C" {
 /* ---- step kernel selection (lb_set_kernel) -------------------------------- */
 #define LB_KERNEL_AUTO 0    /* the fastest kernel for this GPU and lattice: on
                                GB300 overlap for nx >= 1024, else plain, and tiles
-                               instead of strips on smaller lattices              */
+                               instead of strips on smaller lattices, whatever
+                               the strip height                                   */
 #define LB_KERNEL_PLAIN 1   /* coalesced global loads; strips of up to 128 columns
                                (64 threads, two columns each), tiles on smaller
                                lattices unless a strip height was set             */
@@ -141,7 +142,7 @@ int lb_set_replica(lb_ctx *h, uint32_t replica);
 /* Rows of the lattice swept by one CTA of the strip kernels (launch-shape
  * tuning, 1 <= rows <= ny; the default depends on the lattice size; narrow
  * lattices sweep several such bands per CTA).  Does not change results, and has
- * no effect on FP64 lattices, which run in tiles. */
+ * no effect where tiles run: FP64 lattices, and smaller ones under LB_KERNEL_AUTO. */
 int lb_set_strip_height(lb_ctx *h, int rows);
 
 /* Choose the step kernel (LB_KERNEL_*).  All kernels perform the same

@@ -409,7 +409,10 @@ cudaError_t launch_one(lb_ctx *h, int kern, int buf, bool sample, uint32_t step,
     a.wait_ns = h->wait_ns;
     const bool unit = a.gamma == 0.0 && a.gamma_b == 0.0 && a.gamma_g == 0.0;
     a.layout = kern == LB_KERNEL_OVERLAP ? kLayoutWide : kLayoutNarrow;
-    if (h->strip_h == 0 && h->kernel_mode != LB_KERNEL_OVERLAP &&
+    // A strip height asks for strips only where their kernel is asked for too: at 256^2
+    // strips of 8 rows take 11.3 us a step, of 32 rows 32.8, tiles 3.6.
+    if ((h->kernel_mode == LB_KERNEL_AUTO ||
+         (h->kernel_mode != LB_KERNEL_OVERLAP && h->strip_h == 0)) &&
         tile_is_faster(a.nx, a.ny, unit))
         a.layout = kLayoutTile;
     if (h->strip_h > 0) a.strip_h = h->strip_h;

@@ -98,3 +98,18 @@ def test_many_small_residents_at_general_rates():
     for e in es:
         e.close()
     assert general < 1.4 * unit
+
+
+@pytest.mark.parametrize("tau", [1.0, 0.8])
+def test_a_strip_height_leaves_the_automatic_layout(tau):
+    """A height set on a lattice that runs in tiles by itself (strips of 32 rows: 9 times)."""
+    from paper_2212_07848_gb300.lattice import Lattice
+    gs = [Lattice(256, 256, -3.8, tau, 1e-6) for _ in range(2)]
+    for g in gs:
+        g.init(LN2, 5, 1e-3)
+    gs[1].set_strip_height(32)
+    default, tall = _times(gs, [lambda g=g: g.step(64) for g in gs])
+    assert np.array_equal(*(g.download_state() for g in gs))
+    for g in gs:
+        g.close()
+    assert tall < 1.3 * default
