@@ -475,7 +475,8 @@ __device__ __forceinline__ bool mbar_wait_ab(uint64_t *bar, uint32_t parity, uin
 // (tm_xh: 8 channels x 8 pixels, the halo copies); tm_w: the weights as
 // [9][Cout][CIN] with a box of 8 channels x BN output channels (forward only;
 // the input gradient transposes the weights while staging them).
-template <int BN, int CIN, bool DG, bool FOLD>
+// RUNS: a pixel's run of channels leaves from neighbouring lanes.
+template <int BN, int CIN, bool DG, bool FOLD, bool RUNS>
 __global__ void __launch_bounds__(kTcpThreads, 1)
 conv3x3_tcp_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_xh,
                    const __grid_constant__ CUtensorMap tm_w, const bf16 *__restrict__ w,
@@ -800,9 +801,8 @@ conv3x3_tcp_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
                     tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)((t % C::NACC) * BN);
                 constexpr int NQ = CH / 8;   // 16-byte pieces of a pixel's CH channels
                 // lanes that store one pixel's run together: one lane's 16-byte pieces
-                // lie in 32 lines at 64 channels (8 x 512^2, 16 -> 64: 70 us against 114;
-                // 16 -> 32: 53.2 against 55.6; folded 32 -> 32 26.7 without, 28.7 with)
-                constexpr int TR = BN >= 64 || !FOLD ? NQ : 1;
+                // lie in 32 lines at 64 channels (8 x 512^2, 16 -> 64: 70 us against 114)
+                constexpr int TR = RUNS ? NQ : 1;
                 const int sub = lane & (TR - 1);
                 bf16 *yout = y + (((size_t)b * H + row0 + tt) * W + x0 + warp * 32 + lane - sub) * Cout +
                              n0 + sub * 8;
@@ -911,7 +911,7 @@ bool tcp_map_span(CUtensorMap *m, const void *base, uint64_t d0, uint64_t d1, ui
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int BN, int CIN, bool DG, bool FOLD = false>
+template <int BN, int CIN, bool DG, bool FOLD = false, bool RUNS = (BN >= 64)>
 cudaError_t launch_tcp(const bf16 *x, const bf16 *w, const float *bias, bf16 *y, int nb, int h,
                        int wd, int cout, int relu, cudaStream_t s) {
     using C = PCfg<BN, CIN, FOLD>;
@@ -951,9 +951,9 @@ cudaError_t launch_tcp(const bf16 *x, const bf16 *w, const float *bias, bf16 *y,
         if (e == cudaSuccess)
             e = cudaDeviceGetAttribute(&regs_sm, cudaDevAttrMaxRegistersPerMultiprocessor, dev);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(conv3x3_tcp_kernel<BN, CIN, DG, FOLD>,
+            e = cudaFuncSetAttribute(conv3x3_tcp_kernel<BN, CIN, DG, FOLD, RUNS>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-        if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, conv3x3_tcp_kernel<BN, CIN, DG, FOLD>);
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, conv3x3_tcp_kernel<BN, CIN, DG, FOLD, RUNS>);
         if (e != cudaSuccess) {
             nsm = 0;
             return e;
@@ -963,10 +963,18 @@ cudaError_t launch_tcp(const bf16 *x, const bf16 *w, const float *bias, bf16 *y,
     }
     const int nblk = cout / BN;
     const long units = (long)nb * h * (wd / 128);
-    int per_blk = std::max(1, nsm * per_sm / nblk);
-    if (per_blk > units) per_blk = (int)units;
-    const int per = (int)((units + per_blk - 1) / per_blk);
-    conv3x3_tcp_kernel<BN, CIN, DG, FOLD><<<nblk * per_blk, kTcpThreads, kSmem, s>>>(
+    auto ctas = [&](int slots) {   // of an output-channel block
+        return (int)std::min<long>(std::max(1, nsm * slots / nblk), units);
+    };
+    auto rows = [&](int slots) { return (int)((units + ctas(slots) - 1) / ctas(slots)); };
+    // a third slot pays from 16 rows of 128 pixels per SM on, unless the rows divide
+    // over it so badly that an SM gets 3% more of them (16 -> 32: 8 x 128^2, 6.7 rows,
+    // 12.7 us with two and 14.4 with three; 4 x 384^2, 32 rows an SM against 33, 21.3
+    // and 22.0; 8 x 512^2 55.7 and 51.8); with 16 output channels four always do
+    const bool two = BN > 16 && per_sm > 2 &&
+                     (units < 16l * nsm || 103l * 2 * rows(2) <= 100l * per_sm * rows(per_sm));
+    const int slots = two ? 2 : per_sm, per_blk = ctas(slots), per = rows(slots);
+    conv3x3_tcp_kernel<BN, CIN, DG, FOLD, RUNS><<<nblk * per_blk, kTcpThreads, kSmem, s>>>(
         mx, mxh, mw, w, bias, y, nb, h, wd, cout, relu, per_blk, per);
     return cudaGetLastError();
 }
@@ -984,6 +992,10 @@ cudaError_t launch_tcp(const bf16 *x, const bf16 *w, const float *bias, bf16 *y,
 //   the others from 16 rows on (64 -> 64, 27 rows: 49 against 55 us, 6.7 rows 24.6
 //     against 22.6; 128 -> 32, 6.7 rows 32.8 against 31.7; 32 -> 32, 27 rows: 26.7 against 29.2).
 //   16 channels: never (three MMAs a row; 16 -> 16 50 against 45 us at 108 rows).
+// Runs of channels from neighbouring lanes: from 64 output channels on, and 16 -> 32
+// from 16 rows on (108 rows: 51.9 against 58.1 us; 6.7 rows: 11.7 against 10.7); others
+// lose 1 to 8% (32 -> 32 gradient, 10 rows: 16.0 against 15.0 us; 16 -> 16, 243 rows:
+// 76.3 against 74.9).
 template <bool DG>
 cudaError_t launch_tcp_shape(const bf16 *x, const bf16 *w, const float *bias, bf16 *y, int nb,
                              int h, int wd, int cin, int cout, int relu, cudaStream_t s) {
@@ -1001,6 +1013,8 @@ cudaError_t launch_tcp_shape(const bf16 *x, const bf16 *w, const float *bias, bf
     if (WHEN) return launch_tcp<BN, CIN, DG, true>(x, w, bias, y, nb, h, wd, cout, relu, s)
     if (cin == 16) {
         if (cout == 16) TCP(16, 16);
+        if (cout == 32 && many)
+            return launch_tcp<32, 16, DG, false, true>(x, w, bias, y, nb, h, wd, cout, relu, s);
         if (cout == 32) TCP(32, 16);
         if (cout == 64) TCP(64, 16);
         if (cout == 128) TCP(128, 16);
