@@ -1197,7 +1197,10 @@ int lb_ens_autotune(lb_ens *e, int trial_steps, const char *cache_path, int *cho
     ENS_CHECK(cudaGetDeviceProperties(&prop, e->dev));
     std::string key = std::string(prop.name) + "|E" + std::to_string(e->stencil) +
                       (e->launch_mode == LB_ENS_PERSISTENT ? "|P" : "|S") +
-                      (e->ov ? "|ov" : "|hw") + "|R" + std::to_string(e->nres);
+                      // layout and path of the kernel that was timed: a height measured
+                      // for another kernel is not taken
+                      (e->ov ? "|pair128" : "|pair64") + (e->unit ? "|unit" : "|general") +
+                      "|R" + std::to_string(e->nres);
     {
         std::vector<long> sizes;
         for (const auto &q : e->reps) sizes.push_back((long)q.nx * 100000 + q.ny);
