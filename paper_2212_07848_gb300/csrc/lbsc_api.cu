@@ -150,8 +150,7 @@ void fill_base(lb_ctx *h) {
 
 int ensure_io(lb_ctx *h) {
     if (h->d_io) return LB_OK;
-    const size_t n = h->n > 8192 ? h->n : 8192;   // also holds 2 x 4096 radial bins
-    LB_CHECK(cudaMalloc(&h->d_io, n * sizeof(double)));
+    LB_CHECK(cudaMalloc(&h->d_io, h->n * sizeof(double)));   // a density, or the half plane of S(k)
     return LB_OK;
 }
 

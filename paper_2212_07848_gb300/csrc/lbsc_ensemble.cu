@@ -306,7 +306,6 @@ struct lb_ens {
     EnsClock *d_clk = nullptr;
     int *d_flag = nullptr;
     double *d_io = nullptr, *d_partials = nullptr, *d_out = nullptr;
-    size_t io_elems = 0;
     HostReadout rd;                     // radial bins and the flag (lazy, host memory)
     int nred = 0;
     EnsKeys keys;
@@ -852,8 +851,8 @@ int lb_ens_create(lb_ens **out, const lb_replica *reps, int nrep, int psi_kind, 
     if (err == cudaSuccess) err = cudaMalloc(&e->d_reps, nrep * sizeof(EnsRep));
     if (err == cudaSuccess) err = cudaMalloc(&e->d_clk, sizeof(EnsClock));
     if (err == cudaSuccess) err = cudaMalloc(&e->d_flag, sizeof(int));
-    e->io_elems = std::max(max_sites, (size_t)8192);
-    if (err == cudaSuccess) err = cudaMalloc(&e->d_io, e->io_elems * sizeof(double));
+    // a replica's density, or its half plane of S(k)
+    if (err == cudaSuccess) err = cudaMalloc(&e->d_io, max_sites * sizeof(double));
     e->nred = conserved_blocks(4096, 4096);
     if (err == cudaSuccess) err = cudaMalloc(&e->d_partials, 3 * (size_t)e->nred * sizeof(double));
     if (err == cudaSuccess) err = cudaMalloc(&e->d_out, 4 * sizeof(double));
