@@ -442,13 +442,12 @@ def d3q19_leg(n=256, steps=40, strips=(16, 32, 64)):
             "achieved_gbs": gbs, "hbm_frac": gbs / peak, "peak_kind": kind}
 
 
-def l2_assisted_leg(n=1024, steps=2000, strips=(8, 9, 12, 16, 32)):
+def l2_assisted_leg(n=1024, steps=2000):
     """The 1024^2 lattice of the metastable density sweep (FP32, E4, G = -4.5,
     rho0 = 0.33 on the gas branch between coexistence and spinodal, kT =
     1e-6): its 75 MB of populations fit the 129 MB L2, so its rate is
-    L2-assisted and is reported apart from the HBM-bound headline; the
-    fastest of a few strip heights (a 1024^2 lattice fills only about one
-    wave of CTAs, so the strip height decides the halo share and the tail)."""
+    L2-assisted and is reported apart from the HBM-bound headline, as the
+    automatic layout runs it (tiles)."""
     import torch
 
     from paper_2212_07848_gb300.lattice import Lattice
@@ -458,97 +457,77 @@ def l2_assisted_leg(n=1024, steps=2000, strips=(8, 9, 12, 16, 32)):
     lat.sync()
     st = torch.cuda.ExternalStream(lat.stream())
     a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-    best = None
-    for strip in strips:
-        lat.set_strip_height(strip)
-        lat.step(50)
-        a.record(st)
-        lat.step(steps)
-        b.record(st)
-        b.synchronize()
-        t = a.elapsed_time(b) / steps
-        if best is None or t < best[1]:
-            best = (strip, t)
+    lat.step(50)
+    a.record(st)
+    lat.step(steps)
+    b.record(st)
+    b.synchronize()
     lat.close()
-    ms = best[1]
+    ms = a.elapsed_time(b) / steps
     sites = n * n
     # the same lattice as a one-replica ensemble in persistent windows: tiles
     # start a step as soon as their neighbours finished the previous one, so
-    # there is no launch boundary or tail per step
+    # there is no launch boundary or tail per step; at the default height
     from paper_2212_07848_gb300 import abi
     from paper_2212_07848_gb300.ensemble import Ensemble
-    pbest = None
     est = torch.cuda.Stream()
     e = Ensemble([(n, n, -4.5, TAU, KT, 0.33)], seed=SEED, stream=est.cuda_stream)
     e.set_launch(abi.LB_ENS_PERSISTENT)
-    e.set_kernel(abi.LB_KERNEL_OVERLAP)
     e.init(0.0)
-    for strip in (4, 6, 8):
-        e.set_strip_height(strip)
-        e.step(64)
-        e.sync()
-        a.record(est)
-        e.step(steps)
-        b.record(est)
-        b.synchronize()
-        e.sync()
-        t = a.elapsed_time(b) / steps
-        if pbest is None or t < pbest[1]:
-            pbest = (strip, t)
+    e.step(64)
+    e.sync()
+    a.record(est)
+    e.step(steps)
+    b.record(est)
+    b.synchronize()
+    e.sync()
+    pms = a.elapsed_time(b) / steps
     e.close()
-    return {"lattice": f"{n}^2 FP32 E4, G=-4.5, rho0=0.33", "strip_h": best[0], "ms_per_step": ms,
+    return {"lattice": f"{n}^2 FP32 E4, G=-4.5, rho0=0.33", "ms_per_step": ms,
             "mlups": sites / (ms * 1e-3) / 1e6,
             "equivalent_gbs": BYTES_PER_SITE * sites / (ms * 1e-3) / 1e9,
-            "persistent_windows": {"strip_h": pbest[0], "ms_per_step": pbest[1],
-                                   "mlups": sites / (pbest[1] * 1e-3) / 1e6},
+            "persistent_windows": {"ms_per_step": pms, "mlups": sites / (pms * 1e-3) / 1e6},
             "note": "populations (75 MB) resident in L2; not an HBM figure"}
 
 
-def c1_fp64_leg(n=128, steps=2000, sample_from=1001, strips=(1, 2, 4, 8)):
+def c1_fp64_leg(n=128, steps=2000, sample_from=1001):
     """The 128^2 FP64 configuration (psi = 1 - exp(-rho), E4, G = -3.6, rho0 =
     ln 2, tau = 1, kT = 1e-5, seed 0): the whole run, 2000 steps with S(k)
     sampled every step over the last 1000 and the radial read-out, timed
-    with CUDA events for the fastest of a few strip heights, plus the step
-    kernel alone over the first 1000 steps.  144 algorithmic bytes per site
-    (9 FP64 loads + 9 stores); the 2.4 MB of populations stay in L2 and a
-    128^2 lattice gives only 4 to 64 CTAs, so the bound is launch latency and
-    the FP64 pipe, not HBM."""
+    with CUDA events, plus the step kernel alone over the first 1000 steps.
+    144 algorithmic bytes per site (9 FP64 loads + 9 stores); the 2.4 MB of
+    populations stay in L2 and a 128^2 lattice is 128 tiles of 16 x 8 sites,
+    four warps an SM, so the bound is latency and the FP64 pipe, not HBM."""
     import torch
 
     from paper_2212_07848_gb300.lattice import Lattice
-    best = None
     bins = np.empty(n // 2 + 2)
-    for strip in strips:
-        lat = Lattice(n, n, -3.6, 1.0, 1e-5, stencil=4, precision="fp64")
-        lat.set_strip_height(strip)
-        st = torch.cuda.ExternalStream(lat.stream())
-        ev = [torch.cuda.Event(enable_timing=True) for _ in range(3)]
-        for rep in range(2):                      # the first pass warms up
-            lat.init(RHO0, 0, 0.0)
-            lat.sk_config(1, sample_from)
-            lat.sync()
-            ev[0].record(st)
-            lat.step(sample_from - 1)
-            ev[1].record(st)
-            lat.step(steps - sample_from + 1)
-            lat.structure_factor(nbins=len(bins))
-            ev[2].record(st)
-            ev[2].synchronize()
-        lat.close()
-        total = ev[0].elapsed_time(ev[2])
-        plain = ev[0].elapsed_time(ev[1]) / (sample_from - 1)
-        if best is None or total < best[1]:
-            best = (strip, total, plain)
-    strip, total, plain = best
+    lat = Lattice(n, n, -3.6, 1.0, 1e-5, stencil=4, precision="fp64")
+    st = torch.cuda.ExternalStream(lat.stream())
+    ev = [torch.cuda.Event(enable_timing=True) for _ in range(3)]
+    for rep in range(2):                      # the first pass warms up
+        lat.init(RHO0, 0, 0.0)
+        lat.sk_config(1, sample_from)
+        lat.sync()
+        ev[0].record(st)
+        lat.step(sample_from - 1)
+        ev[1].record(st)
+        lat.step(steps - sample_from + 1)
+        lat.structure_factor(nbins=len(bins))
+        ev[2].record(st)
+        ev[2].synchronize()
+    lat.close()
+    total = ev[0].elapsed_time(ev[2])
+    plain = ev[0].elapsed_time(ev[1]) / (sample_from - 1)
     sites = n * n
     peak, kind = _peaks()
     gbs = 144.0 * sites / (plain * 1e-3) / 1e9
-    return {"lattice": f"{n}^2 FP64 E4, G=-3.6, rho0=ln2, kT=1e-5", "strip_h": strip,
+    return {"lattice": f"{n}^2 FP64 E4, G=-3.6, rho0=ln2, kT=1e-5",
             "run_ms": total, "run_mlups": sites * steps / (total * 1e-3) / 1e6,
             "step_ms": plain, "step_mlups": sites / (plain * 1e-3) / 1e6,
             "bytes_per_site": 144, "equivalent_gbs": gbs, "hbm_frac": gbs / peak,
             "peak_kind": kind,
-            "bound": "FP64 arithmetic latency (2.4 MB L2-resident lattice: 128 CTAs of one row, a few warps per SM; steps replayed from captured windows)"}
+            "bound": "FP64 arithmetic latency (2.4 MB L2-resident lattice: 128 tiles of 16 x 8 sites, four warps per SM; steps replayed from captured windows)"}
 
 
 def run_reference(args, rank, world):
