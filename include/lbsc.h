@@ -540,6 +540,12 @@ int lb_nn_mse_channel(const void *y, int c, int ch, const float *target, const f
  * channel 0, 0 elsewhere. */
 int lb_nn_mse(const void *y, int c, const float *target, const float *base, size_t n, float *loss,
               void *dy, void *stream);
+/* The same with a loss that repeats: the squares are added by warps of 32 pixels and
+ * the warps' terms in order, in FP32 (lb_nn_mse adds them as they come).  terms: a
+ * caller-owned device buffer of lb_nn_mse_terms(n) floats. */
+size_t lb_nn_mse_terms(size_t n);
+int lb_nn_mse_ordered(const void *y, int c, const float *target, const float *base, size_t n,
+                      float *loss, float *terms, void *dy, void *stream);
 /* Rollout update: FP32 state [n] += y[.][0] - m, channel 0 of the network
  * input x [n][cx] = BF16(state), channel 2 (when cx > 2) = the increment just
  * applied, other channels of x untouched.  With mean_buf (a caller-owned

@@ -49,7 +49,8 @@ EXPORTED = [
     "lb3_sk_full", "lb3_structure_factor", "lb3_sk_moments",
     "lb_nn_conv3x3", "lb_nn_conv3x3_wgrad", "lb_nn_relu_mask", "lb_nn_pool2", "lb_nn_up2",
     "lb_nn_up2_relu_bwd", "lb_nn_pool2_relu_bwd", "lb_nn_add_up2",
-    "lb_nn_add", "lb_nn_coarse_grain", "lb_nn_mse", "lb_nn_residual", "lb_nn_adam",
+    "lb_nn_add", "lb_nn_coarse_grain", "lb_nn_mse", "lb_nn_mse_terms", "lb_nn_mse_ordered",
+    "lb_nn_residual", "lb_nn_adam",
     "lb_nn_to_bf16", "lb_nn_flux_div", "lb_nn_coarse_momentum", "lb_nn_expand_channel",
     "lb_nn_mse_channel", "lb_nn_mse_blocks", "lb_nn_add_channel", "lb_nn_expand", "lb_nn_wgrad_workspace", "lb_nn_set_conv_path",
     "lb_nn_status", "lb_nn_set_wait_ns",
@@ -198,6 +199,8 @@ def bind(L):
         "lb_nn_add": (C.c_int, [P, P, P, C.c_size_t, P]),
         "lb_nn_coarse_grain": (C.c_int, [P, C.c_int, C.c_int, C.c_int, C.c_double, P, P]),
         "lb_nn_mse": (C.c_int, [P, C.c_int, P, P, C.c_size_t, P, P, P]),
+        "lb_nn_mse_terms": (C.c_size_t, [C.c_size_t]),
+        "lb_nn_mse_ordered": (C.c_int, [P, C.c_int, P, P, C.c_size_t, P, P, P, P]),
         "lb_nn_residual": (C.c_int, [P, P, C.c_int, P, C.c_int, C.c_size_t, P, P]),
         "lb_nn_adam": (C.c_int, [P, P, P, P, P, C.c_size_t, C.c_double, C.c_double, C.c_double,
                                  C.c_double, C.c_longlong, P]),

@@ -783,14 +783,15 @@ __global__ void mse_ch_kernel(const bf16 *__restrict__ y, int C, int ch,
 // VEC (C a multiple of 8, dy 16-byte aligned): a pixel's channels leave as 16-byte
 // stores.  The loss is the FP32 sum of one term per warp (32 terms d^2 added by
 // halves, over n): what a term loses to the running sum's last place depends on the
-// term, so another grouping is another loss in the sixth digit (a term per block: 48
-// us for 68, and losses up to 8e-6 from these).  8 x 512^2, 16 channels: 68 us against
-// 176 us with 2-byte stores; bound by the atomics on one address (8 channels 62 us).
+// term, so another grouping is another loss in the sixth digit.  The terms go to
+// `terms` for an ordered sum (mse_sum_kernel), or are added to the loss as they come.
+// 8 x 512^2, 16 channels: 48 us against 176 us with 2-byte stores, bound by dy's bytes; 68
+// us where they are added, bound by the atomics on one address.
 template <bool VEC>
 __global__ void __launch_bounds__(256)
 mse_kernel(const bf16 *__restrict__ y, int C, const float *__restrict__ tgt,
            const float *__restrict__ base, size_t n, float *__restrict__ loss,
-           bf16 *__restrict__ dy) {
+           float *__restrict__ terms, bf16 *__restrict__ dy) {
     float s = 0.f;
     GRID_STRIDE(i, n) {
         const float d = base[i] + __bfloat162float(y[i * C]) - tgt[i];
@@ -812,7 +813,73 @@ mse_kernel(const bf16 *__restrict__ y, int C, const float *__restrict__ tgt,
         }
     }
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(loss, s / (float)n);
+    if ((threadIdx.x & 31) == 0) {
+        if (terms) terms[(blockIdx.x * 256 + threadIdx.x) >> 5] = s / (float)n;
+        else atomicAdd(loss, s / (float)n);
+    }
+}
+
+// *loss += the terms, one after the other in FP32: the sum that the atomics of a grid
+// in order give, without their scatter (about 1e-6 of the loss).  While the running sum
+// S stays in [C, 2C), C a power of two, every addition rounds its term to a multiple of
+// C's last place, fl(C + a) - C whatever S, so the rounded terms can be added in any
+// order, exactly: eight warps take 256 terms each.  Chunks that take S past 2C, that
+// hold a term half way between two multiples (its rounding depends on S's last bit) or
+// anything that is not finite are added one by one (about ten of the 152 chunks at 8 x
+// 512^2, about 30 us in all; one warp of 512 terms 40 us, all one by one 82 us).
+constexpr int kSumChunk = 256, kSumWarps = 8;
+__global__ void __launch_bounds__(32 * kSumWarps)
+mse_sum_kernel(const float *__restrict__ terms, int n, int padded, float *__restrict__ loss) {
+    constexpr int PER = kSumChunk / 32;
+    extern __shared__ __align__(16) float sh[];   // the terms, zeros from n on
+    __shared__ float s_q[kSumWarps];
+    __shared__ int s_ok[kSumWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll 8
+    for (int k = threadIdx.x; k < padded; k += 32 * kSumWarps) sh[k] = k < n ? terms[k] : 0.f;
+    float S = *loss;   // the same in every thread
+    __syncthreads();
+    for (int pos = 0; pos < padded;) {
+        const float C = __int_as_float(__float_as_int(S) & 0x7f800000);   // 2^e <= S
+        const float half = C * 5.9604644775390625e-8f;                    // C 2^-24
+        const int c0 = pos + warp * kSumChunk;
+        if (c0 < padded) {
+            bool ok = S >= 1e-30f && S <= 1e30f;
+            float q = 0.f;
+#pragma unroll
+            for (int j = 0; j < PER; ++j) {
+                const float a = sh[c0 + 32 * j + lane];
+                const float t = __fadd_rn(C, a), r = __fsub_rn(t, C);
+                ok = ok && a >= 0.f && t < 2.f * C && fabsf(__fsub_rn(a, r)) != half;
+                q = __fadd_rn(q, r);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) q = __fadd_rn(q, __shfl_xor_sync(0xffffffffu, q, o));
+            ok = __all_sync(0xffffffffu, ok);
+            if (lane == 0) {
+                s_q[warp] = q;
+                s_ok[warp] = ok;
+            }
+        }
+        __syncthreads();
+        int k = 0;
+        for (; k < kSumWarps && pos < padded; ++k, pos += kSumChunk) {
+            const float next = __fadd_rn(S, s_q[k]);
+            if (!s_ok[k] || !(next < 2.f * C)) break;
+            S = next;
+        }
+        if (k < kSumWarps && pos < padded) {
+            const float4 *v = reinterpret_cast<const float4 *>(sh + pos);
+#pragma unroll 8
+            for (int j = 0; j < kSumChunk / 4; ++j) {
+                const float4 x = v[j];
+                S = __fadd_rn(__fadd_rn(__fadd_rn(__fadd_rn(S, x.x), x.y), x.z), x.w);
+            }
+            pos += kSumChunk;
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) *loss = S;
 }
 
 // Mean of channel 0 of y [n][C] in two passes with a fixed summation order:
@@ -1188,16 +1255,38 @@ int lb_nn_mse_channel(const void *y, int c, int ch, const float *target, const f
     NN_RET();
 }
 
-int lb_nn_mse(const void *y, int c, const float *target, const float *base, size_t n, float *loss,
-              void *dy, void *stream) {
+static int mse(const void *y, int c, const float *target, const float *base, size_t n, float *loss,
+               float *terms, void *dy, cudaStream_t s) {
     if (!y || !target || !base || !loss || c < 1) return LB_ERR_ARG;
     if (dy && c % 8 == 0 && aligned16(dy, nullptr))
-        mse_kernel<true><<<blocks_for(n), 256, 0, (cudaStream_t)stream>>>(
-            (const bf16 *)y, c, target, base, n, loss, (bf16 *)dy);
+        mse_kernel<true><<<blocks_for(n), 256, 0, s>>>((const bf16 *)y, c, target, base, n, loss,
+                                                       terms, (bf16 *)dy);
     else
-        mse_kernel<false><<<blocks_for(n), 256, 0, (cudaStream_t)stream>>>(
-            (const bf16 *)y, c, target, base, n, loss, (bf16 *)dy);
+        mse_kernel<false><<<blocks_for(n), 256, 0, s>>>((const bf16 *)y, c, target, base, n, loss,
+                                                        terms, (bf16 *)dy);
+    if (terms) {
+        const int count = 8 * blocks_for(n);   // at most 8 x 152 x 32
+        const int padded = (count + kSumChunk - 1) / kSumChunk * kSumChunk;
+        if (cudaGetLastError() != cudaSuccess ||
+            cudaFuncSetAttribute(mse_sum_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 8 * 152 * 32 * (int)sizeof(float)) != cudaSuccess)
+            return LB_ERR_CUDA;
+        mse_sum_kernel<<<1, 32 * kSumWarps, padded * sizeof(float), s>>>(terms, count, padded, loss);
+    }
     NN_RET();
+}
+
+int lb_nn_mse(const void *y, int c, const float *target, const float *base, size_t n, float *loss,
+              void *dy, void *stream) {
+    return mse(y, c, target, base, n, loss, nullptr, dy, (cudaStream_t)stream);
+}
+
+size_t lb_nn_mse_terms(size_t n) { return 8 * (size_t)blocks_for(n); }
+
+int lb_nn_mse_ordered(const void *y, int c, const float *target, const float *base, size_t n,
+                      float *loss, float *terms, void *dy, void *stream) {
+    if (!terms) return LB_ERR_ARG;
+    return mse(y, c, target, base, n, loss, terms, dy, (cudaStream_t)stream);
 }
 
 int lb_nn_residual(float *state, const void *y, int c, void *x, int cx, size_t n, float *mean_buf,

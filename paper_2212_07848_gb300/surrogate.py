@@ -103,6 +103,7 @@ class SurrogateNet:
                  for h, (ci, co) in zip(sizes, LAYERS))
         self.ws_bytes = ws
         self.ws = t.empty(ws // 4, dtype=t.float32, device="cuda")
+        self.loss_terms = t.empty(self.L.lb_nn_mse_terms(nb * n * n), dtype=t.float32, device="cuda")
 
     def _conv(self, x, i, out, relu, h):
         ci, co = LAYERS[i]
@@ -233,8 +234,9 @@ class SurrogateNet:
         npx = nb * n * n
         t0, b0 = (target[0], base[0]) if self.momentum else (target, base)
         d_out = self.dinc if self.flux else self.dy
-        _check(self.L.lb_nn_mse(_p(self.out), self.out_c, _p(t0), _p(b0), npx, _p(loss),
-                                _p(d_out) if grad else None, self.s), "mse")
+        _check(self.L.lb_nn_mse_ordered(_p(self.out), self.out_c, _p(t0), _p(b0), npx, _p(loss),
+                                        _p(self.loss_terms), _p(d_out) if grad else None, self.s),
+               "mse")
         for blk, wgt in self.block_loss:
             _check(self.L.lb_nn_mse_blocks(_p(self.out), self.out_c, _p(t0), _p(b0), nb, n, n, blk,
                                            wgt, _p(loss), _p(d_out) if grad else None, self.s),
