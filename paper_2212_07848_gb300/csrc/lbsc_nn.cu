@@ -281,12 +281,11 @@ wgrad_kernel(const bf16 *__restrict__ x, const bf16 *__restrict__ dy, float *__r
 }
 
 // dw[i] += sum over chunks of part[chunk][i]: a block's eight warps sum every eighth
-// chunk of its 32 V weights and are added in order (a fixed order).  Bound by the
-// partial sums' bytes where there are many weights: then V = 4, a 16-byte load per
-// chunk (64 -> 128: 83 MB in 8.6 us; V = 1 10.6; one thread per weight 13.9.
-// 128 -> 128: 29 MB in 8.9 us; V = 1 18.4).  Where there are few, by the chain of
-// loads: one thread per weight over all chunks left 18 blocks for 16 -> 32 (33.6 us;
-// V = 1 8.6 us).
+// chunk of its 32 V weights and are added in order (a fixed order).  The partial sums
+// were just written and lie in L2.  Many weights: V = 4, a 16-byte load per chunk
+// (64 -> 128: 28 MB in 8.6 us; V = 1 10.6; one thread per weight 13.9.  128 -> 128: 29 MB
+// in 8.9 us; V = 1 18.4).  Few weights are bound by the chain of loads: one thread per
+// weight over all chunks left 18 blocks for 16 -> 32 (33.6 us; V = 1 8.6 us).
 constexpr int kRedWarps = 8;
 template <int V>
 __global__ void __launch_bounds__(32 * kRedWarps)

@@ -28,7 +28,9 @@
 // column per thread at 16 warps an SM, which pulled ten rows for eight and copied
 // the boundary rows every step); 4096 x 32^2: 93 (60).
 // 512 and 768 threads of more registers measured 74; the general path is faster at
-// 512 (63) than at 384 (51).
+// 512 (63) than at 384 (51).  One CTA a replica (C = 1), whose shared-memory loads the
+// compiler interleaves over a thread's pairs, spills 208 bytes a thread at E4 and 256 to
+// 272 at E6 and E8 (general path 480 to 612); the cluster forms none, or 112 to 116.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
