@@ -23,10 +23,11 @@
 // so a resident replica evolves bit-identically to a single lattice with the same
 // seed and replica index.
 //
-// Bound by issue and resident warps: 64^2 on the unit path runs 32 warps an SM at 64
-// registers.  1024 x 64^2: 81 GLUPS (56 with bands of rows swept in lock step, one
-// column per thread at 16 warps an SM, which pulled ten rows for eight and copied
-// the boundary rows every step); 4096 x 32^2: 93 (60).
+// Bound by latency: 64^2 on the unit path runs 32 warps an SM at 64 registers, 214
+// instructions a site update, 46% of the issue slots busy; its warps wait for spilled
+// registers and the shared-memory pipe.  1024 x 64^2: 81 GLUPS (56 with bands of rows
+// swept in lock step, one column per thread at 16 warps an SM, 418 instructions, which
+// pulled ten rows for eight and copied the boundary rows every step); 4096 x 32^2: 93 (60).
 // 512 and 768 threads of more registers measured 74; the general path is faster at
 // 512 (63) than at 384 (51).  One CTA a replica (C = 1), whose shared-memory loads the
 // compiler interleaves over a thread's pairs, spills 208 bytes a thread at E4 and 256 to

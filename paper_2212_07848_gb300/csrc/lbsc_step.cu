@@ -19,8 +19,9 @@
 // from DRAM once per step.  Bound by DRAM at 4096^2 (188 us = 89 GLUPS at 72
 // B/site, 0.95 of the measured copy rate; one column per thread in 128-column
 // strips with scalar arithmetic took 220 us, bound by issue: 391 instructions a
-// site against about 265 now, by the packed FP32 instructions, the shared
-// addresses and the 8-byte accesses) and by issue and resident warps below that.
+// site against 280 now (2048^2, bands of 44 rows), by the packed FP32 instructions,
+// the shared addresses and the 8-byte accesses) and by latency below that (2048^2:
+// 61% of the issue slots, 17 warps an SM, 64% of the DRAM peak).
 // 96 registers (ten 64-thread groups an SM) is the fewest without spills on the
 // unit-relaxation path: eleven and more groups measured 237-290 us, eight 217.
 //
