@@ -822,19 +822,19 @@ mse_kernel(const bf16 *__restrict__ y, int C, const float *__restrict__ tgt,
 // in order give, without their scatter (about 1e-6 of the loss).  While the running sum
 // S stays in [C, 2C), C a power of two, every addition rounds its term to a multiple of
 // C's last place, fl(C + a) - C whatever S, so the rounded terms can be added in any
-// order, exactly: eight warps take 256 terms each.  Chunks that take S past 2C, that
+// order, exactly: sixteen warps take 128 terms each.  Chunks that take S past 2C, that
 // hold a term half way between two multiples (its rounding depends on S's last bit) or
-// anything that is not finite are added one by one (about ten of the 152 chunks at 8 x
-// 512^2, about 30 us in all; one warp of 512 terms 40 us, all one by one 82 us).
-constexpr int kSumChunk = 256, kSumWarps = 8;
+// anything that is not finite are added one by one (about ten of the 304 chunks at 8 x
+// 512^2, about 27 us in all; eight warps of 256 terms 30 us, one warp of 512 40 us, all one by
+// one 82 us).
+constexpr int kSumChunk = 128, kSumWarps = 16;
 __global__ void __launch_bounds__(32 * kSumWarps)
 mse_sum_kernel(const float *__restrict__ terms, int n, int padded, float *__restrict__ loss) {
     constexpr int PER = kSumChunk / 32;
     extern __shared__ __align__(16) float sh[];   // the terms, zeros from n on
-    __shared__ float s_q[kSumWarps];
-    __shared__ int s_ok[kSumWarps];
+    __shared__ __align__(16) float s_q[kSumWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll 8
+#pragma unroll 16
     for (int k = threadIdx.x; k < padded; k += 32 * kSumWarps) sh[k] = k < n ? terms[k] : 0.f;
     float S = *loss;   // the same in every thread
     __syncthreads();
@@ -842,9 +842,9 @@ mse_sum_kernel(const float *__restrict__ terms, int n, int padded, float *__rest
         const float C = __int_as_float(__float_as_int(S) & 0x7f800000);   // 2^e <= S
         const float half = C * 5.9604644775390625e-8f;                    // C 2^-24
         const int c0 = pos + warp * kSumChunk;
+        bool ok = S >= 1e-30f && S <= 1e30f;
+        float q = 0.f;
         if (c0 < padded) {
-            bool ok = S >= 1e-30f && S <= 1e30f;
-            float q = 0.f;
 #pragma unroll
             for (int j = 0; j < PER; ++j) {
                 const float a = sh[c0 + 32 * j + lane];
@@ -852,24 +852,25 @@ mse_sum_kernel(const float *__restrict__ terms, int n, int padded, float *__rest
                 ok = ok && a >= 0.f && t < 2.f * C && fabsf(__fsub_rn(a, r)) != half;
                 q = __fadd_rn(q, r);
             }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) q = __fadd_rn(q, __shfl_xor_sync(0xffffffffu, q, o));
-            ok = __all_sync(0xffffffffu, ok);
-            if (lane == 0) {
-                s_q[warp] = q;
-                s_ok[warp] = ok;
-            }
         }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) q = __fadd_rn(q, __shfl_xor_sync(0xffffffffu, q, o));
+        ok = __all_sync(0xffffffffu, ok);
+        if (lane == 0) s_q[warp] = ok ? q : __int_as_float(0x7f800000);   // infinite: never taken
         __syncthreads();
         int k = 0;
-        for (; k < kSumWarps && pos < padded; ++k, pos += kSumChunk) {
-            const float next = __fadd_rn(S, s_q[k]);
-            if (!s_ok[k] || !(next < 2.f * C)) break;
-            S = next;
+        bool more = true;
+#pragma unroll
+        for (int w = 0; w < kSumWarps; ++w) {
+            const float next = __fadd_rn(S, s_q[w]);
+            more = more && next < 2.f * C;
+            S = more ? next : S;
+            k += more ? 1 : 0;
         }
+        pos += k * kSumChunk;
         if (k < kSumWarps && pos < padded) {
             const float4 *v = reinterpret_cast<const float4 *>(sh + pos);
-#pragma unroll 8
+#pragma unroll 16
             for (int j = 0; j < kSumChunk / 4; ++j) {
                 const float4 x = v[j];
                 S = __fadd_rn(__fadd_rn(__fadd_rn(__fadd_rn(S, x.x), x.y), x.z), x.w);
