@@ -150,7 +150,8 @@ int lb_set_strip_height(lb_ctx *h, int rows);
  * reach the SM and how the pseudopotential halo is exchanged.
  * LB_ERR_UNSUPPORTED if the requested kernel cannot serve the lattice
  * (LB_KERNEL_TMA: FP32 and nx % 128 == 0).
- * lb_get_kernel returns the kernel lb_step uses. */
+ * lb_get_kernel returns the kernel lb_step uses (PLAIN or OVERLAP also where the
+ * lattice runs in tiles instead of their strips). */
 int lb_set_kernel(lb_ctx *h, int mode);
 int lb_get_kernel(const lb_ctx *h);
 

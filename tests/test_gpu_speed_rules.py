@@ -1,5 +1,5 @@
 """Choices of a path whose wrong side costs 1.5 times and more, by the ratio of two calls
-timed in turn on the same device (medians; the limits lie between the two sides)."""
+timed in turn on the same device (the best of nine; the limits lie between the two sides)."""
 import time
 
 import numpy as np
@@ -10,7 +10,7 @@ LN2 = float(np.log(2.0))
 
 
 def _times(objs, calls, rounds=9):
-    """Median seconds of each call, the calls taken in turn."""
+    """Best seconds of each call, the calls taken in turn."""
     got = [[] for _ in calls]
     for k in range(rounds + 2):
         for i, (o, call) in enumerate(zip(objs, calls)):
@@ -20,7 +20,7 @@ def _times(objs, calls, rounds=9):
             o.sync()
             if k >= 2:
                 got[i].append(time.perf_counter() - t)
-    return [sorted(g)[len(g) // 2] for g in got]
+    return [min(g) for g in got]
 
 
 def _ensemble(n, nrep, taus, stencil, launch, resident):
