@@ -284,8 +284,10 @@ wgrad_kernel(const bf16 *__restrict__ x, const bf16 *__restrict__ dy, float *__r
 // chunk of its 32 V weights and are added in order (a fixed order).  The partial sums
 // were just written and lie in L2.  Many weights: V = 4, a 16-byte load per chunk
 // (64 -> 128: 28 MB in 8.6 us; V = 1 10.6; one thread per weight 13.9.  128 -> 128: 29 MB
-// in 8.9 us; V = 1 18.4).  Few weights are bound by the chain of loads: one thread per
-// weight over all chunks left 18 blocks for 16 -> 32 (33.6 us; V = 1 8.6 us).
+// in 8.9 us; V = 1 18.4.  The call of 64 -> 64 at 8 x 64^2, 36864 weights: 29.0 us, V = 1
+// 31.0; 32 -> 64, half as many: no difference).  Few weights are bound by the chain of
+// loads: one thread per weight over all chunks left 18 blocks for 16 -> 32 (33.6 us; V = 1
+// 8.6 us).
 constexpr int kRedWarps = 8;
 template <int V>
 __global__ void __launch_bounds__(32 * kRedWarps)
@@ -1124,7 +1126,7 @@ int lb_nn_conv3x3_wgrad(const void *x, const void *dy, float *dw, float *dbias, 
         if (cudaGetLastError() != cudaSuccess) return LB_ERR_CUDA;
         nchunk = p.nchunk;
     }
-    if (n >= 65536)
+    if (n >= 32768)
         wgrad_reduce_kernel<4><<<(unsigned)(n / 128), 32 * kRedWarps, 0, s>>>(part, dw, n, nchunk);
     else
         wgrad_reduce_kernel<1><<<(unsigned)(n / 32), 32 * kRedWarps, 0, s>>>(part, dw, n, nchunk);
